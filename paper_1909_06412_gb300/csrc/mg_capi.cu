@@ -23,7 +23,8 @@ void* init_tables_kernel(int prec);
 void* obs_tables_kernel(int prec);
 void* set_product_kernel(int prec);
 void* adjoint_kernel(int kind);
-void* short_kernel(int prec, int n, int tma, int tc);
+void* short_kernel(int n, int tma, int tc);
+void* short64_kernel(int n);
 void* regrid_kernel(int prec, int kind);
 void* inner_kernel(int prec);
 int short_threads_for(int prec, int n);
@@ -37,12 +38,13 @@ namespace {
 
 constexpr int MAXBLOCKS = 2048;
 constexpr int RESIDENT_CAP = 96 * 1024;  // bytes per smem region when tiles stay resident
+constexpr int SHORT64_TABLE = 3 * 4096;  // entries of one group multiplier table of the FP64 short-axis kernel
 constexpr int CHUNK_REGION = 64 * 1024;  // bytes per smem region otherwise
 
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
-  size_t ctrl, bar, status, part, tw, tabA, tabAi, tabK, tabV, tabC, tabE, gamma, sct, tabF, tabP, tabB, scratch, total;
+  size_t ctrl, bar, status, part, tw, tabA, tabAi, tabK, tabV, tabC, tabE, gamma, sct, tabF, tabP, tabB, tabT, scratch, total;
 };
 
 // Axis length of a grid the short-axis kernel can take (D >= 3 axes, all of
@@ -88,6 +90,8 @@ Layout layout_for(int D, const int64_t* N, int precision) {
   L.tabF = put(sn ? tt * sizeof(double2) : 0);
   L.tabP = put(sn ? (size_t)(D - 1) * sn * sn * sizeof(double2) : 0);
   L.tabB = put(sn ? 2 * tt * sizeof(double2) : 0);
+  // group multiplier tables of the FP64 short-axis kernel (ShortPlan::tabT, tabQ)
+  L.tabT = put(sn && precision == 0 ? 2 * SHORT64_TABLE * sizeof(int4) : 0);
   L.scratch = put((size_t)npts * (precision == 0 ? sizeof(double2) : sizeof(float2)));
   L.total = o;
   return L;
@@ -229,18 +233,27 @@ void tile_plan(Plan& P) {
 }
 
 // Shared memory of the short-axis kernel for regions of `re` elements: sets
-// region_elems, nreg (3 if it fits, else 2) and smem_bytes.  Must match
-// carve_short() in mg_short.cu.
+// region_elems, nreg (3 if it fits, else 2) and smem_bytes.  FP64 storage:
+// short64_layout() (mg_short.h); FP32 must match carve_short() in mg_short.cu.
 bool short_smem(const Plan& P, ShortPlan& SP, int re) {
+  if (P.prec == 0) {
+    for (int nreg = 3; nreg >= 2; --nreg) {
+      const Short64Layout L = short64_layout(P.D, SP.n, SP.threads, SP.grp[0].g, SP.grp[0].WT, nreg, re);
+      if (L.total > 227 * 1024 - 1024) continue;
+      SP.region_elems = re;
+      SP.nreg = nreg;
+      SP.smem_bytes = L.total;
+      return true;
+    }
+    return false;
+  }
   auto r16 = [](size_t b) { return (b + 15) & ~size_t(15); };
   const size_t tcb = (size_t)short_tc_smem_bytes(SP.tc);
-  const size_t vs = P.prec == 0 ? sizeof(double2) : sizeof(float2);
-  const size_t ts = P.prec == 0 ? sizeof(double) : sizeof(float);
+  const size_t vs = sizeof(float2);
+  const size_t ts = sizeof(float);
   const size_t TT = (size_t)P.tab_total, n = (size_t)SP.n;
-  // the sincos table only for FP64 (the FP32 phases use sincosf); one
-  // 16-value record per warp
-  const size_t tabs = 5 * r16(vs * TT) + (P.prec == 0 ? r16(sizeof(double2) * 256) : 0) +
-                      r16(sizeof(double) * 16 * (size_t)(SP.threads / 32)) + r16(sizeof(double) * PSTRIDE) +
+  // one 16-value record per warp
+  const size_t tabs = 5 * r16(vs * TT) + r16(sizeof(double) * 16 * (size_t)(SP.threads / 32)) + r16(sizeof(double) * PSTRIDE) +
                       r16(sizeof(double) * SCALARS) + r16(sizeof(uint64_t) * 3) + r16(sizeof(unsigned) * 4) +
                       r16(vs * (size_t)(P.D - 1) * n * (n + 1)) + r16(ts * 5 * TT) +
                       r16(vs * (size_t)SP.ngroups * n * (n + 1));
@@ -324,11 +337,19 @@ bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
   SP.n = n;
   SP.ngroups = ngr;
   SP.threads = threads;
+  for (int i = 0; i < ngr; ++i) {
+    SP.toff[i + 1] = SP.toff[i] + SP.grp[i].ng;
+    // 2^s / n^g, and what its rounding left out
+    int s2 = 1;
+    while (2 * s2 <= SP.grp[i].ng) s2 *= 2;
+    const double hi = (double)s2 / SP.grp[i].ng;
+    SP.fscale[i][0] = hi;
+    SP.fscale[i][1] = std::fma(-hi, (double)SP.grp[i].ng, (double)s2) / SP.grp[i].ng;
+  }
+  if (P.prec == 0 && SP.toff[ngr] > SHORT64_TABLE) return false;
   int re = 0;
   for (int i = 0; i < ngr; ++i) re = std::max(re, SP.grp[i].WT * SP.grp[i].PS);
-  if (!short_smem(P, SP, re)) return false;
-  // FP64 12-point lines run two chunks at a time: three regions needed
-  return !(P.prec == 0 && n == 12 && SP.nreg != 3);
+  return short_smem(P, SP, re);
 }
 
 // TMA tensor maps of the short-axis kernel's chunks (FP32 storage, 16-point
@@ -767,7 +788,7 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
   if (!(flags & MG_CREATE_GENERAL_KERNEL) && short_plan(P, c->SP, want_tc)) {
     c->SP.tma = !(flags & MG_CREATE_NO_TMA) && short_tma_maps(P, c->SP, d_psi) ? 1 : 0;
     if (c->SP.tma && !short_tma_smem(P, c->SP)) c->SP.tma = 0;
-    void* fn = short_kernel(P.prec, c->SP.n, c->SP.tma, c->SP.tc);
+    void* fn = P.prec == 0 ? short64_kernel(c->SP.n) : short_kernel(c->SP.n, c->SP.tma, c->SP.tc);
     int occ = 0;
     // the tensor-core variant holds 64 TMEM columns per CTA (512 per SM)
     if (fn && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->SP.smem_bytes) == cudaSuccess &&
@@ -778,6 +799,8 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
       c->SP.tabP = (double2*)(w + L.tabP);
       c->SP.tabB = (double2*)(w + L.tabB);
       c->SP.tabC = c->SP.tabB + P.tab_total;
+      c->SP.tabT = (int4*)(w + L.tabT);
+      c->SP.tabQ = c->SP.tabT + SHORT64_TABLE;
       c->SP.on = 1;
     } else {
       cudaGetLastError();
@@ -1032,7 +1055,7 @@ mg_status mg_propagate(mg_ctx* c, int64_t n_steps, double dt, const char* scheme
   if (short_path) {
     ShortPlan SP = c->SP;
     SP.pairs = c->P.pot_kind == MG_POT_HENON_HEILES;
-    void* sfn = short_kernel(c->P.prec, SP.n, SP.tma, SP.tc);
+    void* sfn = c->P.prec == 0 ? short64_kernel(SP.n) : short_kernel(SP.n, SP.tma, SP.tc);
     void* sargs[] = {&c->P, &B, &R, &SP};
     cudaError_t e = cudaLaunchCooperativeKernel(sfn, dim3(SP.nblocks), dim3(SP.threads), sargs, SP.smem_bytes,
                                                 c->stream);

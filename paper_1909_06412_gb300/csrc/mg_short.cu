@@ -1,6 +1,7 @@
-// Short-axis propagation kernel (sm_103a): the moving-grid split-operator
-// integrator of mg_kernels.cu specialised to tensor grids whose D >= 3 axes
-// all have n = 8, 12 or 16 points (the 8D Henon-Heiles grids of Sec. III.C).
+// Short-axis propagation kernel, FP32 storage (sm_103a): the moving-grid
+// split-operator integrator of mg_kernels.cu specialised to tensor grids whose
+// D >= 3 axes all have n = 8, 12 or 16 points (the 8D Henon-Heiles grids of
+// Sec. III.C).  mg_short64.cu is its counterpart for FP64 storage.
 //
 // Same method and same persistent structure as k_propagate: kinetic substeps
 // U_T,adpt (eq:T_split_substep_adaptive) and potential substeps U_V,adpt
@@ -11,9 +12,8 @@
 //  - A pass transforms a group of up to SHORT_MAXG consecutive axes (mg_short.h),
 //    so a full transform of an 8D grid takes 3-4 passes over the state
 //    instead of 8.
-//  - Chunks are copied between global and shared memory with cp.async
-//    (16 B per FP64 element, 8 B per FP32 element), nreg-1 chunks ahead of the
-//    one being transformed.
+//  - Chunks are copied between global and shared memory with cp.async (8 B
+//    per element), nreg-1 chunks ahead of the one being transformed.
 //  - Each thread transforms whole lines held in registers: an n-point DFT of
 //    compile-time length (8: radix-8 codelet; 12 = 4 x 3 and 16 = 4 x 4 as two
 //    codelet stages with the twiddles in between).
@@ -41,46 +41,20 @@
 #include <stdint.h>
 
 #include "mg_device.cuh"
-#include "mg_short.h"
+#include "mg_short_dev.cuh"
 #include "mg_tc.cuh"
 
 namespace mgk {
 namespace {
 
 // Lines along any group axis per chunk (12-point lines: a multiple of 3) and
-// threads per CTA (one CTA per SM).  FP64 12-point chunks (288 lines = 9
-// warp-sets) go two at a time through 12 warps: the FP64 work spreads over
-// the four SM sub-partitions (5 warp-sets on the busiest against 4.5 on
-// average; one chunk on 9 warps puts 3 on one sub-partition against 2.25),
-// and three warps per sub-partition hide FP64 latency (measured: 12 warps
-// beat 9 by 3.5% and 8 by 7%).  Sixteen warps with 128 registers each spill
-// in the fused passes.
+// threads per CTA (one CTA per SM), for FP32 (prec = 1) and FP64 storage.
 constexpr int short_lpc(int prec, int n) { return n % 3 == 0 ? (prec ? 576 : 288) : (prec ? 512 : 256); }
 // The tensor-core variant (FP32, 16-point lines) holds 256 lines per chunk,
 // one per thread: one round of 128-line GEMMs per warpgroup and axis, and
 // room in shared memory for the operands beside three chunk regions.
 constexpr int short_lpc_tc(int prec, int n, int tc) { return tc ? 256 : short_lpc(prec, n); }
 constexpr int short_threads(int prec, int n) { return n % 3 == 0 ? (prec ? 288 : 384) : 256; }
-
-enum { SM_NONE = 0, SM_KIN = 1, SM_V = 2, SM_VONLY = 3 };
-// scalar slots of the short kernel beyond the shared ones: p before the last
-// potential substep
-constexpr int SC_POLD = 48;
-
-// ---------------------------------------------------------------------------
-// Asynchronous global -> shared copies of one element
-// ---------------------------------------------------------------------------
-
-__device__ __forceinline__ void cp_async_el(double2* s, const double2* g) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_u32(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_async_el(float2* s, const float2* g) {
-  asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_u32(s)), "l"(g) : "memory");
-}
-__device__ __forceinline__ void cp_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
-template <int K> __device__ __forceinline__ void cp_wait() {
-  asm volatile("cp.async.wait_group %0;" ::"n"(K) : "memory");
-}
 
 // ---------------------------------------------------------------------------
 // n-point DFT of a line held in registers (natural order in and out)
@@ -157,67 +131,6 @@ template <bool INV, typename V> struct LineDft<INV, 16, V> {
 };
 
 // ---------------------------------------------------------------------------
-// Per-thread accumulators of the fused reductions
-// ---------------------------------------------------------------------------
-
-template <typename T> struct LineAcc;
-template <> struct LineAcc<double> {
-  double a[MAXD + 1];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int i = 0; i < MAXD + 1; ++i) a[i] = 0.0;
-  }
-  __device__ __forceinline__ void add(int i, double x) { a[i] += x; }
-  __device__ __forceinline__ double get(int i) const { return a[i]; }
-  // i known only at run time: predicated adds keep the array in registers
-  __device__ __forceinline__ void add_rt(int i, double x) {
-#pragma unroll
-    for (int k = 0; k < MAXD + 1; ++k)
-      if (k == i) a[k] += x;
-  }
-  // slot k of o into slot i (known only at run time)
-  __device__ __forceinline__ void merge_rt(int i, const LineAcc& o, int k) { add_rt(i, o.a[k]); }
-};
-template <> struct LineAcc<float> {
-  float s[MAXD + 1], c[MAXD + 1];
-  __device__ __forceinline__ void zero() {
-#pragma unroll
-    for (int i = 0; i < MAXD + 1; ++i) s[i] = c[i] = 0.f;
-  }
-  __device__ __forceinline__ void add(int i, float x) { two_sum_acc(s[i], c[i], x); }
-  __device__ __forceinline__ double get(int i) const { return (double)s[i] + (double)c[i]; }
-  __device__ __forceinline__ void add_rt(int i, float x) {
-#pragma unroll
-    for (int k = 0; k < MAXD + 1; ++k)
-      if (k == i) two_sum_acc(s[k], c[k], x);
-  }
-  __device__ __forceinline__ void merge_rt(int i, const LineAcc& o, int k) {
-    add_rt(i, o.s[k]);
-    add_rt(i, o.c[k]);
-  }
-};
-
-// Sum of acc[0 .. nv-1] over the CTA in a fixed order (warp trees, then warp
-// order) into the CTA's record of `slot`, read back by finish().
-template <typename T>
-__device__ void block_record(const Bufs& B, double* red, int slot, const LineAcc<T>& acc, int nv) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-#pragma unroll
-  for (int v = 0; v < MAXD + 1; ++v)
-    if (v < nv) {
-      const double s = warp_sum(acc.get(v));
-      if (lane == 0) red[warp * 16 + v] = s;
-    }
-  __syncthreads();
-  if (warp == 0 && lane < nv) {
-    double s = 0;
-    for (int w = 0; w < nw; ++w) s += red[w * 16 + lane];
-    __stcg(B.part + ((size_t)slot * gridDim.x + blockIdx.x) * PSTRIDE + lane, s);
-  }
-  __syncthreads();
-}
-
-// ---------------------------------------------------------------------------
 // Shared memory of the short-axis kernel
 // ---------------------------------------------------------------------------
 
@@ -260,9 +173,9 @@ __device__ SSm<V, T> carve_short(const Plan& P, const ShortPlan& SP, unsigned ch
   s.tv = nullptr;
   s.tc = nullptr;
   s.te = nullptr;
-  // the sincos table only for FP64 (expi_prec uses sincosf for FP32); one
-  // 16-value record per warp (block_record)
-  s.sct = P.prec ? nullptr : (double2*)take(sizeof(double2) * 256);
+  // no sincos table (expi_prec uses sincosf for FP32); one 16-value record
+  // per warp (block_record)
+  s.sct = nullptr;
   s.red = (double*)take(sizeof(double) * 16 * (blockDim.x >> 5));
   s.fin = (double*)take(sizeof(double) * PSTRIDE);
   s.sc = (double*)take(sizeof(double) * SC_N);
@@ -305,111 +218,6 @@ __device__ SSm<V, T> carve_short(const Plan& P, const ShortPlan& SP, unsigned ch
   }
   s.end = off;
   return m;
-}
-
-// ---------------------------------------------------------------------------
-// Potential tables: V = sum_a f_a(x_a) + sum_{a<D-1} h_a(x_a) g_{a+1}(x_{a+1})
-// ---------------------------------------------------------------------------
-
-// f, f', g, g', h, h' of axis a at x.
-__device__ __forceinline__ void chain_terms(const Plan& P, int a, double x, double* t) {
-  const int D = P.D;
-  if (P.pot_kind == POT_HENON_HEILES) {
-    const double lam = P.pot[0];
-    t[0] = 0.5 * x * x - (a >= 1 ? lam * x * x * x / 3.0 : 0.0);
-    t[1] = x - (a >= 1 ? lam * x * x : 0.0);
-    t[2] = a >= 1 ? x : 0.0;
-    t[3] = a >= 1 ? 1.0 : 0.0;
-    t[4] = a <= D - 2 ? lam * x * x : 0.0;
-    t[5] = a <= D - 2 ? 2.0 * lam * x : 0.0;
-  } else {  // harmonic with a diagonal force-constant matrix
-    const double k = P.pot[a * D + a];
-    const double d = x - P.pot[D * D + a];
-    t[0] = 0.5 * k * d * d;
-    t[1] = k * d;
-    t[2] = t[3] = t[4] = t[5] = 0.0;
-  }
-}
-
-// Build the per-axis factors F, the gradient columns (in B.tabV) and the pair
-// factors for the grid centred at q_new (scalars SC_QN, SC_SGH of the CTA).
-// Tasks of 32 entries, dealt to warp 0 of every CTA first.  A grid barrier
-// must follow.
-template <typename V>
-__device__ void build_v_short(const Plan& P, const ShortPlan& SP, const Bufs& B, const Smem<V>& S) {
-  const int TT = P.tab_total, n = SP.n;
-  const int nP = SP.pairs ? (P.D - 1) * n * n : 0;
-  const int nchF = (TT + 31) / 32, nchP = (nP + 31) / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const double* sc = S.sc;
-  const double sgh = sc[SC_SGH];
-  for (int t = warp * gridDim.x + blockIdx.x; t < nchF + nchP; t += nwarps * gridDim.x) {
-    if (t < nchF) {
-      const int e = t * 32 + lane;
-      if (e >= TT) continue;
-      const int a = e / n, j = e - a * n;
-      const double x = fma((double)(j - n / 2), P.dq[a], sc[SC_QN + a]);
-      double c[6];
-      chain_terms(P, a, x, c);
-      double sn, cs;
-      expi_prec(P.prec, sgh * c[0], S.sct, sn, cs);
-      __stcg(SP.tabF + e, P.prec ? round_unit_f32(cs, sn, 1.0) : make_double2(cs, sn));
-#pragma unroll
-      for (int k = 0; k < 5; ++k) __stcg(B.tabV + k * TT + e, c[1 + k]);
-    } else {
-      const int e = (t - nchF) * 32 + lane;
-      if (e >= nP) continue;
-      const int a = e / (n * n), rem = e - a * n * n;
-      const int j = rem / n, j2 = rem - j * n;
-      const double x = fma((double)(j - n / 2), P.dq[a], sc[SC_QN + a]);
-      const double y = fma((double)(j2 - n / 2), P.dq[a + 1], sc[SC_QN + a + 1]);
-      double ca[6], cb[6];
-      chain_terms(P, a, x, ca);
-      chain_terms(P, a + 1, y, cb);
-      // the last pair's factor carries the last axis's own term too: the
-      // potential sweep runs along that axis and multiplies by one factor
-      const double th = a == P.D - 2 ? fma(ca[4], cb[2], cb[0]) : ca[4] * cb[2];
-      double sn, cs;
-      expi_prec(P.prec, sgh * th, S.sct, sn, cs);
-      __stcg(SP.tabP + e, P.prec ? round_unit_f32(cs, sn, 1.0) : make_double2(cs, sn));
-    }
-  }
-}
-
-// Multipliers of the forward passes and of the final inverse passes.  Between
-// stages of one launch the stored state carries the demodulation factor of
-// the last kinetic substep, w = A(p) u (A as in mg_kernels.cu), which saves
-// the conj(A)/N multiply of every inverse pass but the last:
-//  - pre  (global SP.tabB, shared tA): A(p)/N_l if the state is u (rel = 0),
-//    else A(p) conj(A(p_old))/N_l = e^{-i (p - p_old) c dq/hbar}/N_l (rel = 1),
-//    with p_old the centre before the last potential substep (SC_POLD);
-//  - post (global SP.tabC, shared tAi): conj(A(p)), applied by the inverse
-//    passes of the launch's last kinetic substep only.
-// The 1/N_l of the unitary pair of transforms sits in the forward multiplier.
-template <typename V>
-__device__ void build_demod_short(const Plan& P, const ShortPlan& SP, const Smem<V>& S, int rel) {
-  const int TT = P.tab_total, n = SP.n;
-  const int nch = (TT + 31) / 32;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
-  const double* sc = S.sc;
-  for (int t = warp * gridDim.x + blockIdx.x; t < 2 * nch; t += nwarps * gridDim.x) {
-    const int e = (t % nch) * 32 + lane;
-    if (e >= TT) continue;
-    const int a = e / n, j = e - a * n;
-    const double c = (double)(j - n / 2);
-    double sn, cs;
-    if (t < nch) {
-      const double dp = rel ? sc[SC_P + a] - sc[SC_POLD + a] : sc[SC_P + a];
-      expi_prec(P.prec, -dp * c * P.dq[a] / P.hbar, S.sct, sn, cs);
-      const double sg = (!rel && (j & 1)) ? -1.0 : 1.0;
-      const double re = sg * cs / (double)n, im = sg * sn / (double)n;
-      __stcg(SP.tabB + e, P.prec ? round_unit_f32(re, im, 1.0 / ((double)n * (double)n)) : make_double2(re, im));
-    } else {
-      expi_prec(P.prec, -sc[SC_P + a] * c * P.dq[a] / P.hbar, S.sct, sn, cs);
-      const double sg = (j & 1) ? -1.0 : 1.0;
-      __stcg(SP.tabC + e, P.prec ? round_unit_f32(sg * cs, -sg * sn, 1.0) : make_double2(sg * cs, -sg * sn));
-    }
-  }
 }
 
 template <typename V>
@@ -459,53 +267,8 @@ __device__ void load_v_short(const Plan& P, const ShortPlan& SP, const Bufs& B, 
 }
 
 // ---------------------------------------------------------------------------
-// Index helpers
-// ---------------------------------------------------------------------------
-
-template <int N> __device__ __forceinline__ int ipow(int k) {
-  int r = 1;
-#pragma unroll
-  for (int i = 0; i < SHORT_MAXG; ++i)
-    if (i < k) r *= N;
-  return r;
-}
-
-// Base-N digits of x into j[a] for lo <= a <= hi (j[hi] least significant).
-template <int N> __device__ __forceinline__ void digits(unsigned x, int lo, int hi, int (&j)[MAXD]) {
-#pragma unroll
-  for (int a = MAXD - 1; a >= 0; --a)
-    if (a >= lo && a <= hi) {
-      const unsigned q = x / N;
-      j[a] = (int)(x - q * N);
-      x = q;
-    }
-}
-
-// j[i] for an index known only at run time, without moving j to local memory.
-__device__ __forceinline__ int pick(const int (&j)[MAXD], int i) {
-  int v = 0;
-#pragma unroll
-  for (int k = 0; k < MAXD; ++k)
-    if (k == i) v = j[k];
-  return v;
-}
-
-// ---------------------------------------------------------------------------
 // Chunk copies
 // ---------------------------------------------------------------------------
-
-// Global offset of chunk c (first element) and its number of planes.
-__device__ __forceinline__ void chunk_geom(const GroupPlan& G, int64_t c, int64_t& gbase, int& nwt) {
-  if (G.contig) {
-    const int64_t b0 = c * G.WT;
-    gbase = b0 * G.ng;
-    nwt = (int)(G.nblk - b0 < G.WT ? G.nblk - b0 : G.WT);
-  } else {
-    const int64_t o = c / G.nb, b = c - o * G.nb;
-    gbase = o * (int64_t)G.ng * G.inner + b * G.WT;
-    nwt = G.WT;
-  }
-}
 
 // Chunk copies, element by element (cp.async in, streaming stores out).  The
 // element index advances by the CTA size each iteration; the chunk
@@ -594,25 +357,6 @@ __device__ __forceinline__ void bulk_wait_read0() { asm volatile("cp.async.bulk.
 __device__ __forceinline__ void bulk_wait_read1() { asm volatile("cp.async.bulk.wait_group.read 1;" ::: "memory"); }
 __device__ __forceinline__ void bulk_wait0() { asm volatile("cp.async.bulk.wait_group 0;" ::: "memory"); }
 __device__ __forceinline__ void fence_proxy_async_all() { asm volatile("fence.proxy.async;" ::: "memory"); }
-
-// Wait for the tensor copies of a chunk, bounded like every wait here: gives
-// up after the barrier time limit (recording MG_ERR_TIMEOUT), or at once when
-// another wait has already failed, so that a failure costs one time limit and
-// not one per chunk.
-__device__ __forceinline__ void wait_chunk(const Bufs& B, uint64_t* bar, unsigned parity) {
-  if (mbar_try_wait(bar, parity)) return;
-  const uint64_t t0 = global_ns();
-  for (unsigned spins = 1;; ++spins) {
-    if (mbar_try_wait(bar, parity)) return;
-    if ((spins & 255u) == 0) {
-      if (*(volatile int*)B.status != ST_OK) return;
-      if (global_ns() - t0 > BARRIER_LIMIT_NS || spins > BARRIER_MAX_SPINS) {
-        atomicExch(B.status, ST_TIMEOUT);
-        return;
-      }
-    }
-  }
-}
 
 // One chunk by tensor copies (issued by one thread).  Group 0: one box of WT
 // whole 16x16x16 blocks.  Strided groups: WT / WP boxes of WP adjacent values of
@@ -717,40 +461,22 @@ __device__ __noinline__ void short_pass(const Plan& P, const ShortPlan& SP, cons
     tmem = *S.tctm;
   }
 
-  // A "set" is the chunk(s) transformed together: one chunk, or two for FP64
-  // 12-point lines (see short_lpc), whose regions rotate X, Y (set) and Z
-  // (prefetch of the next set's first chunk; its second chunk is loaded into
-  // X as soon as the set is stored).
-  constexpr bool PAIR = !TMA && sizeof(T) == 8 && N == 12;
   // prefetch distance: cp.async copies run nreg - 1 chunks ahead; tensor
   // copies one chunk ahead, so that with three regions the next load never
   // waits for the store issued just before it
   const int pd = TMA ? 1 : nreg - 1;
-  int rx = 0, ry = 1, rz = 2;
-  if (PAIR) {
-    for (int s = 0; s < 2; ++s) {
+  for (int s = 0; s < pd; ++s) {
+    if (TMA) {
+      if (threadIdx.x == 0 && s < mine)
+        tma_chunk(SP, G, gi, blockIdx.x + (int64_t)s * gridDim.x, region(S, s), S.s.mbar + s, false);
+    } else {
       if (s < mine) chunk_copy<N, false>(G, psi, blockIdx.x + (int64_t)s * gridDim.x, region(S, s));
       cp_commit();
     }
-  } else {
-    for (int s = 0; s < pd; ++s) {
-      if (TMA) {
-        if (threadIdx.x == 0 && s < mine)
-          tma_chunk(SP, G, gi, blockIdx.x + (int64_t)s * gridDim.x, region(S, s), S.s.mbar + s, false);
-      } else {
-        if (s < mine) chunk_copy<N, false>(G, psi, blockIdx.x + (int64_t)s * gridDim.x, region(S, s));
-        cp_commit();
-      }
-    }
   }
-  for (int64_t i = 0; i < mine; i += PAIR ? 2 : 1) {
+  for (int64_t i = 0; i < mine; ++i) {
     const int ri = (int)(i % nreg);
-    if (PAIR) {
-      if (i + 2 < mine) chunk_copy<N, false>(G, psi, blockIdx.x + (i + 2) * gridDim.x, region(S, rz));
-      cp_commit();
-      cp_wait<1>();
-      __syncthreads();
-    } else {
+    {
       const int64_t i2 = i + pd;
       const int r2 = (int)(i2 % nreg);
       if (TMA) {
@@ -773,23 +499,14 @@ __device__ __noinline__ void short_pass(const Plan& P, const ShortPlan& SP, cons
         __syncthreads();
       }
     }
-    // the set: chunk i (and i+1), its region, lines and first block / index
-    const int ns = (PAIR && i + 1 < mine) ? 2 : 1;
-    V* regs[2];
-    int64_t cs[2];
-    int nls[2];
-    unsigned cbs[2];
-    for (int h = 0; h < 2; ++h) {
-      cs[h] = blockIdx.x + (i + (h < ns ? h : 0)) * gridDim.x;
-      regs[h] = PAIR ? region(S, h ? ry : rx) : region(S, ri);
-      int64_t gb;
-      int nwt;
-      chunk_geom(G, cs[h], gb, nwt);
-      nls[h] = h < ns ? nwt * ipow<N>(g - 1) : 0;  // lines along any group axis
-      // first block (contig) or first trailing index (strided) of the chunk
-      cbs[h] = G.contig ? (unsigned)(cs[h] * G.WT) : (unsigned)((cs[h] % G.nb) * G.WT);
-    }
-    const int nl = nls[0] + nls[1];
+    // the chunk, its region, lines and first block / trailing index
+    const int64_t c = blockIdx.x + i * gridDim.x;
+    V* const reg = region(S, ri);
+    int64_t gb;
+    int nwt;
+    chunk_geom(G, c, gb, nwt);
+    const int nl = nwt * ipow<N>(g - 1);  // lines along any group axis
+    const unsigned cbase = G.contig ? (unsigned)(c * G.WT) : (unsigned)((c % G.nb) * G.WT);
     const int kend = mode == SM_VONLY ? 0 : g;
     for (int kk = 0; kk < kend; ++kk) {
       // forward: last axis of the group first; inverse: first axis first
@@ -813,11 +530,7 @@ __device__ __noinline__ void short_pass(const Plan& P, const ShortPlan& SP, cons
       const int nrounds = (nl + blockDim.x - 1) / blockDim.x;
       for (int Lset = threadIdx.x, rr = 0; TCM != TC_NONE ? rr < nrounds : Lset < nl; Lset += blockDim.x, ++rr) {
         const bool have = TCM == TC_NONE || Lset < nl;
-        const int Lc = have ? Lset : 0;
-        const int hs = Lc >= nls[0];
-        const int L = Lc - (hs ? nls[0] : 0);
-        V* reg = regs[hs];
-        const unsigned cbase = cbs[hs];
+        const int L = have ? Lset : 0;
         int wt, hi, lo, base = 0, stride = 0;
         if (lay == 2) {
           const int t0 = (int)dwp((unsigned)L), w = L - t0 * WP;
@@ -945,11 +658,7 @@ __device__ __noinline__ void short_pass(const Plan& P, const ShortPlan& SP, cons
       // in a sweep of its own: the transform loop above keeps fewer registers live
       const int nhi = ipow<N>(g - 1);
       const Div16 dhi((unsigned)nhi);
-      for (int Lset = threadIdx.x; Lset < nl; Lset += blockDim.x) {
-        const int hs = Lset >= nls[0];
-        const int L = Lset - (hs ? nls[0] : 0);
-        V* reg = regs[hs];
-        const unsigned cbase = cbs[hs];
+      for (int L = threadIdx.x; L < nl; L += blockDim.x) {
         const int wt = (int)dhi((unsigned)L), hi = L - wt * nhi;
         const int base = wt * G.PS + hi * (N + 1);  // padded layout
         const int R = wt * N * N + hi;              // swizzled layout (3-axis block)
@@ -1056,20 +765,12 @@ __device__ __noinline__ void short_pass(const Plan& P, const ShortPlan& SP, cons
       fence_proxy_async();
       __syncthreads();
       if (threadIdx.x == 0) {
-        tma_chunk(SP, G, gi, cs[0], regs[0], nullptr, true);
+        tma_chunk(SP, G, gi, c, reg, nullptr, true);
         bulk_commit();
       }
     } else {
-      for (int h = 0; h < ns; ++h) chunk_copy<N, true>(G, psi, cs[h], regs[h]);
+      chunk_copy<N, true>(G, psi, c, reg);
       __syncthreads();
-      if (PAIR) {
-        if (i + 3 < mine) chunk_copy<N, false>(G, psi, blockIdx.x + (i + 3) * gridDim.x, region(S, rx));
-        cp_commit();
-        const int t = rx;
-        rx = rz;
-        rz = ry;
-        ry = t;
-      }
     }
   }
   if (TMA) {
@@ -1116,7 +817,7 @@ __global__ void __launch_bounds__(short_threads(sizeof(T) == 4, N), 1)
     sc[SC_Q + threadIdx.x] = __ldcg(B.ctrl + threadIdx.x);
     sc[SC_P + threadIdx.x] = __ldcg(B.ctrl + 8 + threadIdx.x);
   }
-  load_tables(P, B, S.s, P.prec ? LT_TW : (LT_TW | LT_SCT));
+  load_tables(P, B, S.s, LT_TW);
   if (TMA) init_mbarriers(S.s);
   // the state enters as u: forward multiplier A/N = conj(conj(A)/N), final
   // post-multiplier conj(A), both exact conversions of the context's tables
@@ -1236,26 +937,23 @@ done:
 // Host-side lookup (C++ linkage, used by mg_capi.cu)
 // ---------------------------------------------------------------------------
 
-// The kernel for FP64 (prec 0) or FP32 (prec 1) storage and axis length n;
+// The kernel for axis length n;
 // tma: the chunk copies use TMA tensor maps (FP32, n = 16 only).
 // tc: the line DFTs on the tensor cores (TC_TF32X3 / TC_BF16X3; FP32, n = 16
 // with TMA only).
-void* short_kernel(int prec, int n, int tma, int tc) {
+void* short_kernel(int n, int tma, int tc) {
   if (tma) {
-    if (prec != 1 || n != 16) return nullptr;
+    if (n != 16) return nullptr;
     // The tensor-core rounds inside this persistent kernel are not enabled:
     // their MMA completions did not arrive (the bounded waits ran out) although
     // the same rounds are exact in a kernel of their own (mg_probe_tc_dft16).
     return tc ? nullptr : (void*)k_propagate_short<float, 16, true, TC_NONE>;
   }
   if (tc) return nullptr;
-  switch (n * 2 + prec) {
-    case 16: return (void*)k_propagate_short<double, 8, false, TC_NONE>;
-    case 17: return (void*)k_propagate_short<float, 8, false, TC_NONE>;
-    case 24: return (void*)k_propagate_short<double, 12, false, TC_NONE>;
-    case 25: return (void*)k_propagate_short<float, 12, false, TC_NONE>;
-    case 32: return (void*)k_propagate_short<double, 16, false, TC_NONE>;
-    case 33: return (void*)k_propagate_short<float, 16, false, TC_NONE>;
+  switch (n) {
+    case 8: return (void*)k_propagate_short<float, 8, false, TC_NONE>;
+    case 12: return (void*)k_propagate_short<float, 12, false, TC_NONE>;
+    case 16: return (void*)k_propagate_short<float, 16, false, TC_NONE>;
   }
   return nullptr;
 }

@@ -67,6 +67,13 @@ struct ShortPlan {
   double2* tabC;     // [D*n] post-multiplier conj(A) of a launch's last inverse passes
   double2* tabF;     // [D*n] e^{-i sigma f_a(x)/hbar} per axis entry
   double2* tabP;     // [(D-1)*n*n] e^{-i sigma h_a(x_a) g_{a+1}(x_{a+1})/hbar}
+  // FP64 kernel: multipliers of every point of a group's n^g block, in the
+  // form of mg_fixed.cuh: tabT before the transforms of a pass, tabQ after
+  // those of a launch's last inverse passes; group gi starts at toff[gi]
+  int4* tabT;
+  int4* tabQ;
+  int toff[MAXD + 1];
+  double fscale[MAXD][2];  // 2^s / n^g of each group as hi + lo, s = floor(log2 n^g)
   // TMA (tma = 1): one tensor map per group over psi.  The group that ends at
   // the last axis is a rank-4 view {n, n, n, blocks} (innermost first) copied
   // in boxes of {n, n, n, WT} with the 128-byte swizzle; a strided group is a
@@ -74,5 +81,49 @@ struct ShortPlan {
   // boxes of {WP, n, .., 1}, WP = min(WT, 256), WT / WP boxes per chunk.
   TensorMapBytes tmap[MAXD];
 };
+
+#ifdef __CUDACC__
+#define MG_HD __host__ __device__
+#else
+#define MG_HD
+#endif
+
+// Shared memory of the FP64 short-axis kernel (mg_short64.cu) as byte
+// offsets, used by the planner and by the kernel.
+struct Short64Layout {
+  int F, Pt, col, Gh, U, Lo, pc, jl, es, cd, red, fin, sc, mbar, mphase, reg, total;
+};
+constexpr int SHORT64_PC = 10;  // doubles of a plane's potential record
+
+MG_HD inline Short64Layout short64_layout(int D, int n, int threads, int g0, int WT0, int nreg, int region_elems) {
+  Short64Layout L{};
+  int o = 0;
+  const int TT = D * n;
+  int ng1 = 1;
+  for (int k = 1; k < g0; ++k) ng1 *= n;
+  auto put = [&](int bytes) {
+    const int at = o;
+    o = (o + bytes + 15) & ~15;
+    return at;
+  };
+  L.F = put(16 * TT);
+  L.Pt = put(16 * (D - 1) * n * (n + 1));
+  L.col = put(8 * 5 * TT);
+  L.Gh = put(16 * ng1);
+  L.U = put(8 * 4 * ng1);
+  L.Lo = put(16 * 2 * WT0);
+  L.pc = put(8 * SHORT64_PC * 2 * WT0);
+  L.jl = put(4 * 2 * WT0);
+  L.es = put(4 * 2 * 16);
+  L.cd = put(8 * (n + 2));
+  L.red = put(8 * 16 * (threads / 32));
+  L.fin = put(8 * PSTRIDE);
+  L.sc = put(8 * SCALARS);
+  L.mbar = put(8 * 3);
+  L.mphase = put(16);
+  L.reg = o;
+  L.total = o + nreg * 16 * region_elems;
+  return L;
+}
 
 }  // namespace mgk
