@@ -279,7 +279,7 @@ bool short_smem(const Plan& P, ShortPlan& SP, int re) {
 // most axes whose blocks tile a chunk; the other groups, from the back, the
 // most axes (up to SHORT_MAXG) whose chunk rows of WT adjacent elements are
 // at least 32 bytes (one DRAM sector) and divide the trailing index range.
-bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
+bool short_plan_lpc(const Plan& P, ShortPlan& SP, int tc, int lpc) {
   std::memset(&SP, 0, sizeof(ShortPlan));
   SP.tc = tc;
   const int D = P.D;
@@ -287,7 +287,6 @@ bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
   if (!n || P.minv_general) return false;  // per-axis kinetic tables only
   const size_t vs = P.prec == 0 ? sizeof(double2) : sizeof(float2);
   const int threads = short_threads_for(P.prec, n);
-  const int lpc = short_lpc_for(P.prec, n, tc);
   auto pw = [&](int k) {
     int64_t r = 1;
     for (int i = 0; i < k; ++i) r *= n;
@@ -350,6 +349,43 @@ bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
   int re = 0;
   for (int i = 0; i < ngr; ++i) re = std::max(re, SP.grp[i].WT * SP.grp[i].PS);
   return short_smem(P, SP, re);
+}
+
+// The plan with the chunk size that suits the grid (FP32 chunks have one size).
+// A pass is bound by latency, not by throughput: measured, a warp takes about
+// 4000 cycles for its lines of one axis whether it shares its scheduler with
+// none or two others, a chunk about 8000 for its copies and waits, and 3000
+// stand for the barrier of a pass.  So a grid with fewer chunks than teams
+// (two per SM) gains from smaller chunks, even at more passes, and a large one
+// keeps the largest.  Microseconds per kinetic unit with the largest chunks
+// and with the ones chosen: 12^4 126 (288 lines) -> 96 (144); 12^5 137 (288) ->
+// 106 (144); 16^4 137 (256) -> 100 (32); 8^4 94 (256) -> 74 (64); 12^3 69 -> 66;
+// 16^5 and larger keep theirs.
+bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
+  const int n = short_shape(P.D, P.N);
+  if (!n) return false;
+  const int full = short_lpc_for(P.prec, n, tc);
+  if (P.prec != 0) return short_plan_lpc(P, SP, tc, full);
+  constexpr int64_t TEAMS_ALL = 2 * 152;
+  double best = 0;
+  bool ok = false;
+  for (int d = 1; full / d >= n; ++d) {
+    ShortPlan C;
+    if (full % d || !short_plan_lpc(P, C, tc, full / d)) continue;
+    double cost = 0;
+    for (int i = 0; i < C.ngroups; ++i) {
+      const GroupPlan& G = C.grp[i];
+      const int64_t waves = (G.nchunks + TEAMS_ALL - 1) / TEAMS_ALL;
+      const int lines = full / d, team = C.threads / 2, rounds = (lines + team - 1) / team;
+      cost += (double)waves * (4.0 * G.g * rounds + 8.0) + 3.0;
+    }
+    if (!ok || cost < best) {
+      best = cost;
+      SP = C;
+      ok = true;
+    }
+  }
+  return ok;
 }
 
 // TMA tensor maps of the short-axis kernel's chunks (FP32 storage, 16-point
