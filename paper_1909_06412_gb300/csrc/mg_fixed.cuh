@@ -337,6 +337,12 @@ __host__ __device__ __forceinline__ long long to_fixed(int hi, unsigned lo, int 
   return ((long long)v ^ s) - s;
 }
 #ifdef __CUDACC__
+// An infinity or NaN, which multiplier words cannot carry: where a phase
+// overflows its table entries are NaN, the kernel notes it in SC_BAD and ends
+// with the status that the FP64 sums of such a state give.
+constexpr int SC_BAD = 37;
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+__device__ __forceinline__ bool not_finite(double2 v) { return not_finite(v.x) || not_finite(v.y); }
 __device__ __forceinline__ I2 to_fixed2(double2 v, int ref) {
   return I2{to_fixed(__double2hiint(v.x), (unsigned)__double2loint(v.x), ref),
             to_fixed(__double2hiint(v.y), (unsigned)__double2loint(v.y), ref)};

@@ -106,7 +106,7 @@ constexpr double M61 = 2305843009213693952.0;  // 2^61
 // must follow.
 enum { GT_U = 0, GT_REL = 1, GT_K = 2, GT_POST = 3 };
 template <int N>
-__device__ void build_group_table(const Plan& P, const ShortPlan& SP, const double* sc, const double2* sct, int kind,
+__device__ void build_group_table(const Plan& P, const ShortPlan& SP, double* sc, const double2* sct, int kind,
                                   int4* dst) {
   const int total = SP.toff[SP.ngroups], nch = (total + 31) / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
@@ -141,8 +141,15 @@ __device__ void build_group_table(const Plan& P, const ShortPlan& SP, const doub
       cs = -cs;
       sn = -sn;
     }
+    if (not_finite(make_double2(cs, sn))) sc[SC_BAD] = 1.0;
     __stcg(dst + e, to_mult(make_double2(cs, sn), M61));
   }
+}
+
+__device__ __forceinline__ double2 load_factor(const double2* t, double* sc) {
+  const double2 f = __ldcg(t);
+  if (not_finite(f)) sc[SC_BAD] = 1.0;
+  return f;
 }
 
 // Last axis along a line: g = g0 + g1 rho, f' = c0 + c1 rho + c2 rho^2, g' and
@@ -178,12 +185,12 @@ __device__ __forceinline__ LastAxis last_axis(const Plan& P, double x, double dq
 template <int N> __device__ void load_v64(const Plan& P, const ShortPlan& SP, const Bufs& B, const S64& S) {
   const int TT = P.tab_total, D = P.D;
   for (int e = threadIdx.x; e < TT; e += blockDim.x) {
-    S.F[e] = to_mult(__ldcg(SP.tabF + e), M61);
+    S.F[e] = to_mult(load_factor(SP.tabF + e, S.s.sc), M61);
 #pragma unroll
     for (int k = 0; k < 5; ++k) S.col[k * TT + e] = __ldcg(B.tabV + k * TT + e);
   }
   for (int e = threadIdx.x; e < (D - 1) * N * N; e += blockDim.x) {
-    if (SP.pairs) S.Pt[e + e / N] = to_mult(__ldcg(SP.tabP + e), M61);
+    if (SP.pairs) S.Pt[e + e / N] = to_mult(load_factor(SP.tabP + e, S.s.sc), M61);
     else if (e >= (D - 2) * N * N) S.Pt[e + e / N] = to_mult(__ldcg(SP.tabF + (D - 1) * N + e % N), M61);
   }
   const int g = SP.grp[0].g, l0 = SP.grp[0].l0;
@@ -746,6 +753,7 @@ done:
     }
     if (sc[SC_ERR] != 0.0) atomicExch(B.status, (int)sc[SC_ERR]);
   }
+  if (threadIdx.x == 0 && sc[SC_BAD] != 0.0) atomicExch(B.status, ST_NONFINITE);
 }
 
 }  // namespace
