@@ -216,8 +216,14 @@ done:
   }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(THREADS, 1) k_batch(const __grid_constant__ BatchArgs BA) {
+// CTAS per SM.  A team spends most of a pass waiting for copies, barriers and
+// short dependent chains, and a second CTA's team fills that; with half the
+// registers each is slower by itself.  512 uneven 2D and 3D grids, FP32, two
+// suzuki4 steps: 51.6 ms with one CTA of up to 255 registers a thread, 34.5 ms
+// with two of 128 (spills of about 1 KB a thread); a batch that one CTA per SM
+// takes in one go is 8% faster that way (the host's rule, mg_batch_create).
+template <typename T, int CTAS>
+__global__ void __launch_bounds__(THREADS, CTAS) k_batch(const __grid_constant__ BatchArgs BA) {
   using V = typename VT<T>::v;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ Plan sP;
@@ -253,6 +259,9 @@ __global__ void __launch_bounds__(THREADS, 1) k_batch(const __grid_constant__ Ba
 
 }  // namespace
 
-void* batch_kernel(int prec) { return prec ? (void*)k_batch<float> : (void*)k_batch<double>; }
+void* batch_kernel(int prec, int ctas) {
+  if (ctas == 2) return prec ? (void*)k_batch<float, 2> : (void*)k_batch<double, 2>;
+  return prec ? (void*)k_batch<float, 1> : (void*)k_batch<double, 1>;
+}
 
 }  // namespace mgk

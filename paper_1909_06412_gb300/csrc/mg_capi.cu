@@ -1681,7 +1681,7 @@ extern "C" mg_status mg_propagate_noalloc(int D, const int64_t* N, const double*
 // ---------------------------------------------------------------------------
 
 namespace mgk {
-void* batch_kernel(int prec);
+void* batch_kernel(int prec, int ctas);
 }
 
 namespace {
@@ -1890,11 +1890,6 @@ mg_status mg_batch_create(mg_batch** out, int nprob, mg_ctx* const* ctxs, int cl
   }
   b->smem = A.smem_bytes;
 
-  void* fn = batch_kernel(prec);
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, A.smem_bytes) != cudaSuccess) {
-    delete b;
-    return MG_ERR_CUDA;
-  }
   cudaLaunchAttribute attr[1];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = cluster;
@@ -1906,10 +1901,26 @@ mg_status mg_batch_create(mg_batch** out, int nprob, mg_ctx* const* ctxs, int cl
   cfg.dynamicSmemBytes = A.smem_bytes;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
+  // one CTA per SM when its teams take every problem at once, else the kernel
+  // that runs two (where the shared memory of two fits)
+  void* fn = nullptr;
   int ncl = 0;
-  if (cudaOccupancyMaxActiveClusters(&ncl, fn, &cfg) != cudaSuccess || ncl < 1) {
-    delete b;
-    return MG_ERR_UNSUPPORTED;
+  for (int ctas = 1; ctas <= 2; ++ctas) {
+    void* f = batch_kernel(prec, ctas);
+    int n = 0;
+    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, A.smem_bytes) != cudaSuccess) {
+      delete b;
+      return MG_ERR_CUDA;
+    }
+    if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess || n < 1) {
+      delete b;
+      return MG_ERR_UNSUPPORTED;
+    }
+    if (n > ncl) {
+      fn = f;
+      ncl = n;
+    }
+    if (nprob <= ncl) break;
   }
   b->nteams = std::min(std::min(ncl, nprob), MAXTEAMS);
   A.nteams = b->nteams;
