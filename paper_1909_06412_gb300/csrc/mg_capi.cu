@@ -609,6 +609,7 @@ struct mg_ctx {
   double stuck_barrier_s;  // test hook: > 0 arms a barrier that cannot complete (mg_test_stuck_barrier)
   int64_t launches;
   std::vector<double> host;  // staging for psi
+  std::vector<double> back;  // mg_get_observables' read-back
   std::vector<double> gam;
   double ctrl[32];
 };
@@ -650,18 +651,29 @@ mg_status init_tables(mg_ctx* c) {
 
 mg_status refresh_tables(mg_ctx* c) { return c->tables_stale ? init_tables(c) : MG_OK; }
 
-mg_status read_status(mg_ctx* c) {
-  cudaError_t e = cudaStreamSynchronize(c->stream);
+// Waits for the stream and reads back the first `bytes` of the workspace: the
+// control block, the status word and the reductions' records lie one behind
+// the other (layout_for), so that one copy serves a call that needs several.
+// A pending device status is cleared and returned.
+mg_status read_back(mg_ctx* c, void* host, size_t bytes) {
+  cudaError_t e = cudaMemcpyAsync(host, c->d_work, bytes, cudaMemcpyDeviceToHost, c->stream);
+  if (e == cudaSuccess) e = cudaStreamSynchronize(c->stream);
   if (e != cudaSuccess) return MG_ERR_CUDA;
   int st = 0;
-  e = cudaMemcpy(&st, c->B.status, sizeof(int), cudaMemcpyDeviceToHost);
-  if (e != cudaSuccess) return MG_ERR_CUDA;
+  std::memcpy(&st, (const char*)host + c->L.status, sizeof(int));
   if (st != 0) {
     int zero = 0;
     cudaMemcpy(c->B.status, &zero, sizeof(int), cudaMemcpyHostToDevice);
     return (mg_status)st;
   }
   return MG_OK;
+}
+
+constexpr size_t HEAD_BYTES = 1024;  // control block, barrier words, status
+
+mg_status read_status(mg_ctx* c) {
+  char head[HEAD_BYTES];
+  return read_back(c, head, c->L.status + sizeof(int));
 }
 
 double sqrt_cell(const Plan& P) {
@@ -1218,11 +1230,11 @@ mg_status mg_sync(mg_ctx* c) {
 mg_status mg_get_state(mg_ctx* c, double* psi, double* q, double* p, double* t) {
   if (!c) return MG_ERR_ARG;
   if (!c->state_set) return MG_ERR_STATE;
-  mg_status s = read_status(c);
+  alignas(16) char head[HEAD_BYTES];
+  mg_status s = read_back(c, head, c->L.status + sizeof(int));
   if (s != MG_OK) return s;
   const int D = c->P.D;
-  double ctrl[17];
-  if (cudaMemcpy(ctrl, c->B.ctrl, sizeof(ctrl), cudaMemcpyDeviceToHost) != cudaSuccess) return MG_ERR_CUDA;
+  const double* ctrl = (const double*)head;  // the control block comes first
   for (int a = 0; a < D; ++a) {
     c->q[a] = ctrl[a];
     c->p[a] = ctrl[8 + a];
@@ -1248,11 +1260,9 @@ mg_status mg_get_state(mg_ctx* c, double* psi, double* q, double* p, double* t) 
 mg_status mg_get_observables(mg_ctx* c, double* norm, double* energy, double* mean_q, double* mean_p) {
   if (!c) return MG_ERR_ARG;
   if (!c->state_set || !c->pot_set) return MG_ERR_STATE;
-  mg_status s = read_status(c);
-  if (s != MG_OK) return s;
   const Plan& P = c->P;
   void* targs[] = {&c->P, &c->B};
-  s = refresh_tables(c);
+  mg_status s = refresh_tables(c);
   if (s == MG_OK) s = launch_plain(c, obs_tables_kernel(P.prec), targs, P.smem_bytes);
   void* fn = obs_kernel(P.prec, P.pot_kind);
   for (int l = P.D - 1; l >= 0 && s == MG_OK; --l) {
@@ -1266,15 +1276,14 @@ mg_status mg_get_observables(mg_ctx* c, double* norm, double* energy, double* me
     s = launch_plain(c, fn, args, P.smem_bytes);
   }
   if (s != MG_OK) return s;
-  s = read_status(c);
+  // a status pending from before the call is reported here too
+  const int nb = P.nblocks, D = P.D;
+  const size_t part_bytes = 2ull * nb * PSTRIDE * sizeof(double);
+  c->back.resize((c->L.part + part_bytes) / sizeof(double));
+  s = read_back(c, c->back.data(), c->L.part + part_bytes);
   if (s != MG_OK) return s;
-  const int nb = P.nblocks;
-  std::vector<double> part(2ull * nb * PSTRIDE);
-  if (cudaMemcpy(part.data(), c->B.part, part.size() * sizeof(double), cudaMemcpyDeviceToHost) != cudaSuccess)
-    return MG_ERR_CUDA;
-  double ctrl[17];
-  if (cudaMemcpy(ctrl, c->B.ctrl, sizeof(ctrl), cudaMemcpyDeviceToHost) != cudaSuccess) return MG_ERR_CUDA;
-  const int D = P.D;
+  const double* ctrl = c->back.data();
+  const double* part = c->back.data() + c->L.part / sizeof(double);
   double k[PSTRIDE] = {0}, v[PSTRIDE] = {0};
   for (int b = 0; b < nb; ++b)
     for (int i = 0; i < D + 2; ++i) {
