@@ -18,6 +18,7 @@
 
 namespace mgk {
 void* propagate_kernel(int prec, int kind);
+void* propagate64_kernel(int kind, int D);
 void* obs_kernel(int prec, int kind);
 void* init_tables_kernel(int prec);
 void* obs_tables_kernel(int prec);
@@ -84,7 +85,7 @@ Layout layout_for(int D, const int64_t* N, int precision) {
   L.tabC = put(tt * sizeof(double));
   L.tabE = put(tt * sizeof(double));
   L.gamma = put(MAX_STAGES * sizeof(double));
-  L.sct = put(256 * sizeof(double2));
+  L.sct = put(sizeof(double2) * 256 + sizeof(int4) * 512);
   // per-axis and pair potential factors of the short-axis kernel
   const int sn = short_shape(D, N);
   L.tabF = put(sn ? tt * sizeof(double2) : 0);
@@ -131,7 +132,7 @@ size_t smem_for(const Plan& P) {
   const int nmult = (P.tab_global & TG_MULT) ? 0 : 3;
   const int ncols = (P.tab_global & TG_COLS) ? 0 : 1;
   size_t s = (1 + nmult) * r16(vs * TT) + ncols * (r16(sizeof(double) * NVCOL * TT) + 2 * r16(sizeof(double) * TT)) +
-             r16(sizeof(double2) * 256) + r16(sizeof(double) * THREADS * (3 * P.D + 5)) +
+             r16(sizeof(double2) * (P.fixed64 ? 512 : 256)) + r16(sizeof(double) * THREADS * (3 * P.D + 5)) +
              r16(sizeof(double) * PSTRIDE) + r16(sizeof(double) * SCALARS) +
              (P.resident ? 2 : 3) * r16((size_t)P.region_bytes) + r16(sizeof(uint64_t) * 3) +
              r16(sizeof(unsigned) * 4) + r16(sizeof(int64_t) * P.max_tiles) +
@@ -230,6 +231,32 @@ void tile_plan(Plan& P) {
   if (P.smem_bytes <= SMEM_CAP || P.prec != 0) return;
   P.tab_global = TG_COLS | TG_MULT;
   tile_plan_tables(P);
+}
+
+// Plan of k_propagate64 in place of P's kernel, for FP64 grids with enough
+// points.  The integer passes have the higher throughput and the longer
+// latency for a few points (one CTA per SM either way): measured per yoshida4
+// call 1.39x on 128^3 (13,800 points per SM) and 1.17x on 128 x 2048 (1725),
+// 0.89x on 256^2 (431) and 0.80x on 32^3 (216); the line is drawn between.
+constexpr int64_t FIXED64_POINTS = 1024;  // per SM
+
+bool plan64(const Plan& P, int sms, Plan& Q) {
+  if (P.prec != 0 || P.npts < FIXED64_POINTS * sms) return false;
+  Q = P;
+  Q.fixed64 = 1;
+  Q.nblocks = sms;
+  tile_plan(Q);
+  if (Q.smem_bytes > SMEM_CAP) return false;
+  for (int kind = 0; kind < 4; ++kind) {
+    void* fn = propagate64_kernel(kind, Q.D);
+    int occ = 0;
+    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Q.smem_bytes) != cudaSuccess ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, Q.smem_bytes) != cudaSuccess || occ < 1) {
+      cudaGetLastError();
+      return false;
+    }
+  }
+  return true;
 }
 
 // Shared memory of the short-axis kernel for regions of `re` elements: sets
@@ -560,6 +587,38 @@ void fill_sincos_table(double* t) {
   }
 }
 
+// The two tables of rotate_turns (mg_pass64.cuh): e^{2 pi i k / 256} and
+// e^{2 pi i k / 65536} as multiplier words (scale 2^61), rounded from the
+// extended-precision value; 512 x 4 ints.
+void fill_phase_words(int* t) {
+  for (int k = 0; k < 512; ++k) {
+    const long double a = 2.0L * 3.14159265358979323846264338327950288L * (long double)(k & 255) /
+                          (k < 256 ? 256.0L : 65536.0L);
+    const long long c = llroundl(std::cos(a) * 2305843009213693952.0L);
+    const long long s = llroundl(std::sin(a) * 2305843009213693952.0L);
+    t[4 * k] = (int)(c >> 31);
+    t[4 * k + 1] = (int)(c & 0x7fffffff);
+    t[4 * k + 2] = (int)(s >> 31);
+    t[4 * k + 3] = (int)(s & 0x7fffffff);
+  }
+}
+
+// Both tables as they lie in a workspace (Layout::sct), computed once per
+// process: the extended-precision functions take longer than the rest of
+// mg_create.
+struct PhaseTables {
+  double sct[512];
+  int words[2048];
+  PhaseTables() {
+    fill_sincos_table(sct);
+    fill_phase_words(words);
+  }
+};
+const PhaseTables& phase_tables() {
+  static const PhaseTables t;
+  return t;
+}
+
 // Forward twiddles e^{-2 pi i m / n}, m = 0 .. n-1, into t (2 n doubles):
 // correctly rounded FP64 pairs, or for FP32 storage the float pairs of
 // round_unit_f32_host.
@@ -597,6 +656,7 @@ double digamma(double x) {
 
 struct mg_ctx {
   Plan P;
+  Plan P64;      // plan of k_propagate64 (fixed64 = 0 when P's kernel propagates)
   ShortPlan SP;  // short-axis kernel plan (SP.on = 0 when the grid does not qualify)
   Bufs B;
   Layout L;
@@ -622,6 +682,15 @@ mg_status cuda_ok(cudaError_t e) { return e == cudaSuccess ? MG_OK : MG_ERR_CUDA
 // the ones the short-axis kernel evaluates from per-axis and pair tables.
 bool uses_short_kernel(const Plan& P) {
   return P.pot_kind == MG_POT_HENON_HEILES || (P.pot_kind == MG_POT_HARMONIC && !P.pot_general);
+}
+
+// The general kernel's plan for the context's current potential.
+Plan& general_plan(mg_ctx* c) {
+  if (!c->P64.fixed64) return c->P;
+  c->P64.pot_kind = c->P.pot_kind;
+  c->P64.pot_general = c->P.pot_general;
+  std::memcpy(c->P64.pot, c->P.pot, sizeof(c->P.pot));
+  return c->P64;
 }
 
 mg_status upload_ctrl(mg_ctx* c) {
@@ -830,7 +899,14 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
   B.tabE = (double*)(w + L.tabE);
   B.gamma = (const double*)(w + L.gamma);
   B.sct = (double2*)(w + L.sct);
+  B.words = (int4*)(B.sct + 256);
   B.scratch = (double2*)(w + L.scratch);
+
+  c->P64.fixed64 = 0;
+  {
+    Plan Q;
+    if (plan64(P, std::min(MAXBLOCKS, sms), Q)) c->P64 = Q;
+  }
 
   // short-axis kernel: one CTA per SM, all co-resident
   if (!(flags & MG_CREATE_GENERAL_KERNEL) && short_plan(P, c->SP, want_tc)) {
@@ -869,10 +945,9 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
     fill_twiddles(n, P.prec, &tw[2 * P.ax[l].toff]);
     for (int m = 0; m < n; ++m) kc[P.ax[l].toff + m] = (double)(m - n / 2);
   }
-  std::vector<double> sct(512);
-  fill_sincos_table(sct.data());
+  const PhaseTables& pt = phase_tables();
   mg_status s = cuda_ok(cudaMemsetAsync(d_work, 0, L.scratch, c->stream));
-  if (s == MG_OK) s = cuda_ok(cudaMemcpyAsync(B.sct, sct.data(), 512 * sizeof(double), cudaMemcpyHostToDevice, c->stream));
+  if (s == MG_OK) s = cuda_ok(cudaMemcpyAsync(B.sct, &pt, sizeof(pt), cudaMemcpyHostToDevice, c->stream));
   if (s == MG_OK) s = cuda_ok(cudaMemcpyAsync(B.tw, tw.data(), tw.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   if (s == MG_OK) s = cuda_ok(cudaMemcpyAsync(B.tabC, kc.data(), kc.size() * sizeof(double), cudaMemcpyHostToDevice, c->stream));
   if (s == MG_OK) s = cuda_ok(cudaStreamSynchronize(c->stream));
@@ -1093,7 +1168,7 @@ mg_status mg_propagate(mg_ctx* c, int64_t n_steps, double dt, const char* scheme
     // test hook: the barrier word starts with gridDim.x arrivals of the
     // current generation, so no arrival is ever the last one; every CTA's
     // wait runs out after the short limit and the kernel returns
-    const unsigned long long word = (unsigned long long)(short_path ? c->SP.nblocks : c->P.nblocks);
+    const unsigned long long word = (unsigned long long)(short_path ? c->SP.nblocks : general_plan(c).nblocks);
     s = cuda_ok(cudaMemcpyAsync(c->B.bar, &word, sizeof(word), cudaMemcpyHostToDevice, c->stream));
     if (s == MG_OK) s = cuda_ok(cudaStreamSynchronize(c->stream));
     if (s != MG_OK) return s;
@@ -1112,13 +1187,14 @@ mg_status mg_propagate(mg_ctx* c, int64_t n_steps, double dt, const char* scheme
     c->t += (double)n_steps * dt;
     return MG_OK;
   }
-  void* fn = propagate_kernel(c->P.prec, c->P.pot_kind);
+  Plan& G = general_plan(c);
+  void* fn = G.fixed64 ? propagate64_kernel(c->P.pot_kind, c->P.D) : propagate_kernel(c->P.prec, c->P.pot_kind);
   if (!fn) return MG_ERR_UNSUPPORTED;
-  if (c->P.smem_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->P.smem_bytes) != cudaSuccess)
+  if (G.smem_bytes > 48 * 1024 &&
+      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G.smem_bytes) != cudaSuccess)
     return MG_ERR_CUDA;
-  void* args[] = {&c->P, &B, &R};
-  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(c->P.nblocks), dim3(THREADS), args, c->P.smem_bytes, c->stream);
+  void* args[] = {&G, &B, &R};
+  cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(G.nblocks), dim3(THREADS), args, G.smem_bytes, c->stream);
   c->launches++;
   if (e != cudaSuccess) return MG_ERR_CUDA;
   c->t += (double)n_steps * dt;
@@ -1630,8 +1706,8 @@ extern "C" mg_status mg_propagate_noalloc(int D, const int64_t* N, const double*
   // The array keeps the previous call's contents: the barrier words and the
   // status word must start at zero; every other table is rewritten before use.
   cudaStream_t st = (cudaStream_t)cuda_stream;
-  double tw[2 * NOALLOC_MAXTAB], kc[NOALLOC_MAXTAB], ctrl[17], sct[512];
-  fill_sincos_table(sct);
+  double tw[2 * NOALLOC_MAXTAB], kc[NOALLOC_MAXTAB], ctrl[17];
+  const double(&sct)[512] = phase_tables().sct;
   for (int l = 0; l < D; ++l) {
     const int n = P.ax[l].n;
     fill_twiddles(n, MG_FP64, &tw[2 * P.ax[l].toff]);
@@ -1975,14 +2051,12 @@ mg_status mg_batch_create(mg_batch** out, int nprob, mg_ctx* const* ctxs, int cl
   A.dt = (const double*)(w + L.run + sizeof(BatchRun));
   A.bstatus = (int*)(w + L.bstatus);
   A.sct = (const double2*)(w + L.sct);
-  std::vector<double> sct(512);
-  fill_sincos_table(sct.data());
   b->run_bytes = sizeof(BatchRun) + (size_t)nprob * sizeof(double);
   mg_status s = cuda_ok(cudaMemcpy(w + L.probs, b->hprob.data(), sizeof(BatchProb) * nprob, cudaMemcpyHostToDevice));
   if (s == MG_OK) s = cuda_ok(cudaMemcpy(w + L.team_start, start.data(), start.size() * sizeof(int), cudaMemcpyHostToDevice));
   if (s == MG_OK) s = cuda_ok(cudaMemcpy(w + L.team_items, items.data(), items.size() * sizeof(int), cudaMemcpyHostToDevice));
   if (s == MG_OK) s = cuda_ok(cudaMemset(w + L.bstatus, 0, (size_t)nprob * sizeof(int)));
-  if (s == MG_OK) s = cuda_ok(cudaMemcpy(w + L.sct, sct.data(), 512 * sizeof(double), cudaMemcpyHostToDevice));
+  if (s == MG_OK) s = cuda_ok(cudaMemcpy(w + L.sct, phase_tables().sct, 512 * sizeof(double), cudaMemcpyHostToDevice));
   if (s == MG_OK) s = cuda_ok(cudaHostAlloc((void**)&b->h_run, b->run_bytes, cudaHostAllocDefault));
   if (s == MG_OK) std::memset(b->h_run, 0, b->run_bytes);
   if (s == MG_OK) s = cuda_ok(cudaEventCreateWithFlags(&b->done, cudaEventDisableTiming));

@@ -377,7 +377,7 @@ template <typename V> __device__ Smem<V> carve(const Plan& P, const Bufs& B, uns
     s.tc = (double*)take(sizeof(double) * TT);
     s.te = (double*)take(sizeof(double) * TT);
   }
-  s.sct = (double2*)take(sizeof(double2) * 256);
+  s.sct = (double2*)take(sizeof(double2) * (P.fixed64 ? 512 : 256));
   s.red = (double*)take(sizeof(double) * THREADS * (3 * P.D + 5));
   s.fin = (double*)take(sizeof(double) * PSTRIDE);
   s.sc = (double*)take(sizeof(double) * SC_N);

@@ -150,6 +150,9 @@ __host__ __device__ __forceinline__ void idft4(I2& v0, I2& v1, I2& v2, I2& v3, L
 
 // 1 - sqrt(3)/2, 1/(2 sqrt(2)) and 1/(4 sqrt(2)), times 2^63
 constexpr int C3H = 575416509, C3L = 516773425;
+// 1 - pi/4 and 1/3, times 2^63 (rotate_turns)
+constexpr int C1MPI4H = 921707869, C1MPI4L = 1867226854;
+constexpr int C13H = 1431655765, C13L = 715827883;
 constexpr int C4H = 1518500249, C4L = 2121767201;
 constexpr int C8H = 759250124, C8L = 2134625425;
 

@@ -32,6 +32,7 @@
 #include <stdint.h>
 
 #include "mg_device.cuh"
+#include "mg_pass64.cuh"
 
 namespace mgk {
 namespace {
@@ -40,9 +41,16 @@ namespace {
 // The persistent propagation kernel
 // ---------------------------------------------------------------------------
 
-template <typename T, int KIND>
-__global__ void __launch_bounds__(THREADS, 1)
-    k_propagate(const __grid_constant__ Plan P, const __grid_constant__ Bufs B, const __grid_constant__ Run RN) {
+struct Forward {
+  static constexpr bool value = false;
+};
+struct Inverse {
+  static constexpr bool value = true;
+};
+
+// F64: the passes of axis_pass64 (FP64 storage), else those of axis_pass.
+template <typename T, int KIND, bool F64, int DM = MAXD>
+__device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, const Run& RN) {
   using V = typename VT<T>::v;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sflag;
@@ -57,7 +65,23 @@ __global__ void __launch_bounds__(THREADS, 1)
     sc[SC_Q + threadIdx.x] = __ldcg(B.ctrl + threadIdx.x);
     sc[SC_P + threadIdx.x] = __ldcg(B.ctrl + 8 + threadIdx.x);
   }
-  load_tables(P, B, S, LT_TW | LT_A | LT_C | LT_SCT);
+  // passes on the integer units: tables in multiplier form, phases in turns
+  Smem<V> SB = S;  // for the table builds, which use the FP64 sincos table
+  if (F64) SB.sct = (double2*)B.sct;
+  auto load = [&](int what) {
+    if constexpr (F64) load_mult_tables(P, B, S, what);
+    else load_tables(P, B, S, what);
+  };
+  auto pass = [&](auto inv, const PassArgs& a, int r) {
+    if constexpr (F64) return axis_pass64<decltype(inv)::value, KIND, DM>(P, B, a, r);
+    else return axis_pass<T, decltype(inv)::value, KIND>(P, B, a, S, r);
+  };
+  auto phase_scale = [&](double sig) {
+    const double x = -sig / P.hbar;
+    if constexpr (F64) return turns_scale(x, sc);
+    else return x;
+  };
+  load(LT_TW | LT_A | LT_C | LT_SCT);
   init_mbarriers(S);
   const double* gam = B.gamma;
   int res = -1;
@@ -67,26 +91,26 @@ __global__ void __launch_bounds__(THREADS, 1)
     if (threadIdx.x == 0) {
       const double sig = (RN.split == SPLIT_VTV ? 0.5 : 1.0) * gam[0] * RN.dt;
       sc[SC_SIG] = sig;
-      sc[SC_SGH] = -sig / P.hbar;
+      sc[SC_SGH] = phase_scale(sig);
     }
     if (threadIdx.x < D) sc[SC_QN + threadIdx.x] = sc[SC_Q + threadIdx.x];
     __syncthreads();
-    build_tables(P, B, S, TB_V);
+    build_tables(P, B, SB, TB_V);
     if (!grid_sync(B, &sflag)) return;
-    load_tables(P, B, S, LT_V);
+    load(LT_V);
     __syncthreads();
     PassArgs a{};
     a.l = D - 1; a.fft = 0; a.red = RED_V; a.slot = 1;
     a.keep = P.resident; a.src = B.psi; a.dst = B.psi;
-    res = axis_pass<T, false, KIND>(P, B, a, S, -1);
+    res = pass(Forward{}, a, -1);
     kept = P.resident;
     if (!grid_sync(B, &sflag)) return;
     finish(B, S, 1, D + 1);
     centre_after_potential(P, S, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
-    build_tables(P, B, S, TB_A);
+    build_tables(P, B, SB, TB_A);
     if (!grid_sync(B, &sflag)) return;
-    load_tables(P, B, S, LT_A);
+    load(LT_A);
     __syncthreads();
   }
 
@@ -97,7 +121,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       unit_coeffs(RN, gam, u, tau, sig, hasv);
       sc[SC_TAU] = tau;
       sc[SC_SIG] = sig;
-      sc[SC_SGH] = -sig / P.hbar;
+      sc[SC_SGH] = phase_scale(sig);
       sc[SC_HASV] = hasv ? 1.0 : 0.0;
     }
     __syncthreads();
@@ -111,7 +135,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       a.keep = last && P.resident;
       a.red = last ? RED_KIN : RED_NONE; a.slot = 0;
       a.src = B.psi; a.dst = B.psi;
-      res = axis_pass<T, false, KIND>(P, B, a, S, res);
+      res = pass(Forward{}, a, res);
       kept = a.keep;
       if (!last && !grid_sync(B, &sflag)) return;
     }
@@ -119,9 +143,9 @@ __global__ void __launch_bounds__(THREADS, 1)
     finish(B, S, 0, D + 1);
     centre_after_kinetic(P, S, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
-    build_tables(P, B, S, TB_K | (hasv ? TB_V : 0));
+    build_tables(P, B, SB, TB_K | (hasv ? TB_V : 0));
     if (!grid_sync(B, &sflag)) return;
-    load_tables(P, B, S, LT_K | (hasv ? LT_V : 0));
+    load(LT_K | (hasv ? LT_V : 0));
     if (threadIdx.x < D) sc[SC_Q + threadIdx.x] = sc[SC_QN + threadIdx.x];
     __syncthreads();
     // inverse transform, potential substep fused into the last pass
@@ -133,7 +157,7 @@ __global__ void __launch_bounds__(THREADS, 1)
       a.keep = last && hasv && P.resident;
       a.red = (last && hasv) ? RED_V : RED_NONE; a.slot = 1;
       a.src = B.psi; a.dst = B.psi;
-      res = axis_pass<T, true, KIND>(P, B, a, S, res);
+      res = pass(Inverse{}, a, res);
       kept = a.keep;
       if (!last && !grid_sync(B, &sflag)) return;
     }
@@ -142,9 +166,9 @@ __global__ void __launch_bounds__(THREADS, 1)
       finish(B, S, 1, D + 1);
       centre_after_potential(P, S, RN.motion);
       if (sc[SC_ERR] != 0.0) goto done;
-      build_tables(P, B, S, TB_A);
+      build_tables(P, B, SB, TB_A);
       if (!grid_sync(B, &sflag)) return;
-      load_tables(P, B, S, LT_A);
+      load(LT_A);
       __syncthreads();
     }
   }
@@ -157,6 +181,18 @@ done:
     }
     if (sc[SC_ERR] != 0.0) atomicExch(B.status, (int)sc[SC_ERR]);
   }
+  if (F64 && threadIdx.x == 0 && sc[SC_BAD] != 0.0) atomicExch(B.status, ST_NONFINITE);
+}
+
+template <typename T, int KIND>
+__global__ void __launch_bounds__(THREADS, 1)
+    k_propagate(const __grid_constant__ Plan P, const __grid_constant__ Bufs B, const __grid_constant__ Run RN) {
+  propagate_body<T, KIND, false>(P, B, RN);
+}
+template <int KIND, int DM>
+__global__ void __launch_bounds__(THREADS, 1)
+    k_propagate64(const __grid_constant__ Plan P, const __grid_constant__ Bufs B, const __grid_constant__ Run RN) {
+  propagate_body<double, KIND, true, DM>(P, B, RN);
 }
 
 // Tables A/Ainv for the current p-centre (after a state upload).  The
@@ -273,6 +309,18 @@ void* propagate_kernel(int prec, int kind) {
     case POT_ATOM_DIATOM * 2 + 1: return prop_fn<float, POT_ATOM_DIATOM>();
     case POT_HENON_HEILES * 2 + 1: return prop_fn<float, POT_HENON_HEILES>();
     case POT_SECREST_JOHNSON * 2 + 1: return prop_fn<float, POT_SECREST_JOHNSON>();
+  }
+  return nullptr;
+}
+
+// FP64 storage with the passes on the integer units (Plan::fixed64), for D axes.
+void* propagate64_kernel(int kind, int D) {
+  switch (kind) {
+    case POT_HARMONIC: return D <= 3 ? (void*)k_propagate64<POT_HARMONIC, 3> : (void*)k_propagate64<POT_HARMONIC, MAXD>;
+    case POT_ATOM_DIATOM: return (void*)k_propagate64<POT_ATOM_DIATOM, 2>;
+    case POT_HENON_HEILES:
+      return D <= 3 ? (void*)k_propagate64<POT_HENON_HEILES, 3> : (void*)k_propagate64<POT_HENON_HEILES, MAXD>;
+    case POT_SECREST_JOHNSON: return (void*)k_propagate64<POT_SECREST_JOHNSON, 2>;
   }
   return nullptr;
 }

@@ -42,6 +42,7 @@ struct Plan {
   int D;
   int prec;              // 0 = FP64, 1 = FP32 storage
   int nblocks;           // CTAs of the persistent kernel (all co-resident)
+  int fixed64;           // plan of k_propagate64 (FP64 passes on the integer units, mg_pass64.cuh)
   int resident;          // tiles of axes 0 and D-1 stay in smem across barriers
   int maxn;              // longest axis
   int tab_total;         // sum of N_l
@@ -77,6 +78,7 @@ struct Bufs {
   double* tabE;          // per-axis kinetic energy minv_l (p_l^K)^2 / 2
   const double* gamma;   // composition coefficients
   double2* sct;          // 256 entries e^{i k pi / 128}
+  int4* words;           // the tables of rotate_turns (mg_pass64.cuh)
   double2* scratch;      // npts complex128 (observables, host staging)
   uint64_t bar_limit_ns; // time limit of a grid-barrier wait (0 = the default 5 s)
 };
