@@ -333,17 +333,24 @@ __host__ __device__ __forceinline__ BlockScale block_scale(int E, unsigned Y, in
 __host__ __device__ __forceinline__ long long to_fixed(int hi, unsigned lo, int ref) {
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
   const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 10;
-  int sh = ref - (int)(((unsigned)hi >> 20) & 0x7ffu);
-  sh = sh > 63 ? 63 : sh;
+  // above 63 the value is zero; below zero only for a value above the bound
+  // (an infinity or NaN as a multiplier, which its reader notes: SC_BAD)
+  unsigned sh = (unsigned)(ref - (int)(((unsigned)hi >> 20) & 0x7ffu));
+  sh = sh > 63u ? 63u : sh;
   const unsigned long long v = (m >> sh) & ~1ull;
   const long long s = (long long)(hi >> 31);
   return ((long long)v ^ s) - s;
 }
 #ifdef __CUDACC__
 // An infinity or NaN, which multiplier words cannot carry: where a phase
-// overflows its table entries are NaN, the kernel notes it in SC_BAD and ends
-// with the status that the FP64 sums of such a state give.
+// overflows its table entries are NaN.  Whoever turns such an entry into words
+// notes it in its CTA's SC_BAD, and in word BAR_BAD of the launch's barrier
+// block if other CTAs read the words.  From then on its passes write NaN, as
+// the products with the entry would be, and its next sum, NaN too, ends the
+// launch.
 constexpr int SC_BAD = 37;
+constexpr int BAR_BAD = 32;
+__device__ __forceinline__ bool noted_bad(const double* sc) { return __double2hiint(sc[SC_BAD]) != 0; }
 __device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 __device__ __forceinline__ bool not_finite(double2 v) { return not_finite(v.x) || not_finite(v.y); }
 __device__ __forceinline__ I2 to_fixed2(double2 v, int ref) {

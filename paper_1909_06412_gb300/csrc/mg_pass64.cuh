@@ -37,7 +37,9 @@ __device__ __forceinline__ int4 mult_bits(double2 v, int s) {
 // floor(log2 n): conj(A)/n is held times 2^this
 __device__ __forceinline__ int post_shift(int n) { return 31 - __clz(n); }
 
-// The per-axis tables in multiplier form (in place of load_tables' FP64 pairs).
+// The per-axis tables in multiplier form (in place of load_tables' FP64
+// pairs).  Entries that stay in the workspace are turned into words, and
+// checked, where a pass reads them.
 __device__ void load_mult_tables(const Plan& P, const Bufs& B, const Smem<double2>& S, int what) {
   const int TT = P.tab_total;
   load_tables(P, B, S, what & ~(LT_TW | LT_A | LT_K | LT_SCT));
@@ -122,11 +124,11 @@ __device__ __forceinline__ I2 rotate_turns(I2 x, double t, float eps, const int4
 // One Stockham pass of radix R over L lines of length n (see stockham_pass),
 // divided by 2^SC.  The first pass (Ns == 1) converts its FP64 inputs at the
 // chunk's scale and applies `pre` (shared) or `preg` (FP64 entries in the
-// workspace).
+// workspace; one that is not finite is noted in `bad`).
 template <bool INV, int R, int SC>
 __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* __restrict__ out, int n, int L,
                                                 Div16 divL, int Ns, const int4* tw, const int4* pre,
-                                                const double2* preg, int wsh, int ref) {
+                                                const double2* preg, int wsh, int ref, double* bad) {
   const int nR = n / R;
   const int total = L * nR;
   const int ts = n / (Ns * R);
@@ -170,7 +172,11 @@ __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* _
         for (int r = 0; r < R; ++r) v[r] = cmul<false, true>(v[r], pre[j + r * nR]);
       } else if (preg) {
 #pragma unroll
-        for (int r = 0; r < R; ++r) v[r] = cmul<false, true>(v[r], mult_bits(__ldcg(preg + j + r * nR), 0));
+        for (int r = 0; r < R; ++r) {
+          const double2 m = __ldcg(preg + j + r * nR);
+          if (not_finite(m)) *bad = 1.0;
+          v[r] = cmul<false, true>(v[r], mult_bits(m, 0));
+        }
       }
     }
     const LineBits lb = line_bits(v[0], v[1]);
@@ -202,7 +208,7 @@ __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* _
 // (radix 2, 4, 8: sqrt(R); radix 3 counted as 2).
 template <bool INV>
 __device__ I2* stockham64(I2* in, I2* out, int L, const AxisPlan& ax, const int4* tw, const int4* pre,
-                          const double2* preg, int wsh, int ref, int& eo) {
+                          const double2* preg, int wsh, int ref, double* bad, int& eo) {
   int Ns = 1, h = 0;
   const int n = ax.n;
   const Div16 divL((unsigned)L);
@@ -213,15 +219,15 @@ __device__ I2* stockham64(I2* in, I2* out, int L, const AxisPlan& ax, const int4
     h &= 1;
     eo += sc;
     if (R == 8) {
-      if (sc == 1) stockham64_pass<INV, 8, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
-      else stockham64_pass<INV, 8, 2>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
+      if (sc == 1) stockham64_pass<INV, 8, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
+      else stockham64_pass<INV, 8, 2>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
     } else if (R == 4) {
-      stockham64_pass<INV, 4, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
+      stockham64_pass<INV, 4, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
     } else if (R == 3) {
-      stockham64_pass<INV, 3, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
+      stockham64_pass<INV, 3, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
     } else {
-      if (sc == 0) stockham64_pass<INV, 2, 0>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
-      else stockham64_pass<INV, 2, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref);
+      if (sc == 0) stockham64_pass<INV, 2, 0>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
+      else stockham64_pass<INV, 2, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
     }
     __syncthreads();
     I2* t = in;
@@ -386,10 +392,11 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
     int eo = bs.eo;
     I2* ic = (I2*)cur;
     if (A.fft) {
-      ic = stockham64<INV>(ic, (I2*)oth, nt * W, ax, tw, pre, preg, wsh, bs.ref, eo);
+      ic = stockham64<INV>(ic, (I2*)oth, nt * W, ax, tw, pre, preg, wsh, bs.ref, S.sc + SC_BAD, eo);
       cur = (V*)ic;
     }
     if (postT) eo -= post_shift(n);
+    const bool poison = bs.poison || noted_bad(S.sc);
 
     // epilogue: element e of the chunk is tile ti, point j, line w
     for (int e = threadIdx.x; e < cnt; e += blockDim.x) {
@@ -399,7 +406,21 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
       const int j = contig ? rem - w * n : rem >> wsh;
       I2 x = ic[e];
       if (!A.fft) x = I2{to_fixed(hi32(x.x), (unsigned)x.x, bs.ref), to_fixed(hi32(x.y), (unsigned)x.y, bs.ref)};
-      if (postT) x = cmul<false, true>(x, gmult ? mult_bits(__ldcg(postT + j), post_shift(n)) : ((const int4*)postT)[j]);
+      bool nan = poison;
+      if (postT) {
+        int4 m;
+        if (gmult) {
+          const V f = __ldcg(postT + j);
+          if (not_finite(f)) {
+            nan = true;
+            S.sc[SC_BAD] = 1.0;
+          }
+          m = mult_bits(f, post_shift(n));
+        } else {
+          m = ((const int4*)postT)[j];
+        }
+        x = cmul<false, true>(x, m);
+      }
       V v;
       if (A.red != RED_NONE) {
         int idx[DM];
@@ -409,7 +430,7 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
         idx[A.l] = j;
         if (A.red == RED_KIN) {
           v = from_fixed2(x, eo);
-          const double w2 = bs.poison ? __longlong_as_double(0x7ff8000000000000ll) : fma(v.x, v.x, v.y * v.y);
+          const double w2 = nan ? __longlong_as_double(0x7ff8000000000000ll) : fma(v.x, v.x, v.y * v.y);
           acc[0] += w2;
 #pragma unroll
           for (int a = 0; a < DM; ++a)
@@ -418,6 +439,7 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
             // the non-separable part of the kinetic phase (see axis_pass)
             const double th = over_hbar(P, -S.sc[SC_TAU] * kinetic_cross<DM>(P, S.tc, S.sc, idx));
             v = from_fixed2(rotate_turns(x, th * INV_2PI, KIN_TEPS, tab), eo);
+            nan = nan || not_finite(th);
           }
         } else {  // RED_V
           double th, g[DM];
@@ -425,8 +447,8 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
           // |x|^2 is the same before and after the phase
           v = from_fixed2(rotate_turns(x, th, teps, tab), eo);
           // an overflowing potential leaves no phase: a NaN, as its sine would be
-          if (not_finite(th)) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
-          const double w2 = bs.poison ? __longlong_as_double(0x7ff8000000000000ll) : fma(v.x, v.x, v.y * v.y);
+          nan = nan || not_finite(th);
+          const double w2 = nan ? __longlong_as_double(0x7ff8000000000000ll) : fma(v.x, v.x, v.y * v.y);
           acc[0] += w2;
 #pragma unroll
           for (int a = 0; a < DM; ++a)
@@ -435,7 +457,7 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
       } else {
         v = from_fixed2(x, eo);
       }
-      if (bs.poison) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
+      if (nan) v.x = v.y = __longlong_as_double(0x7ff8000000000000ll);
       if (A.keep) cur[e] = v;
       else if (dst) __stcg(dst + S.tb[ti] + j * es + w * ws, v);
     }

@@ -113,8 +113,7 @@ constexpr double M61 = 2305843009213693952.0;  // 2^61
 // must follow.
 enum { GT_U = 0, GT_REL = 1, GT_K = 2, GT_POST = 3 };
 template <int N>
-__device__ void build_group_table(const Plan& P, const ShortPlan& SP, double* sc, const double2* sct, int kind,
-                                  int4* dst) {
+__device__ void build_group_table(const Plan& P, const ShortPlan& SP, const Bufs& B, double* sc, int kind, int4* dst) {
   const int total = SP.toff[SP.ngroups], nch = (total + 31) / 32;
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarps = blockDim.x >> 5;
   for (int t = warp * gridDim.x + blockIdx.x; t < nch; t += nwarps * gridDim.x) {
@@ -137,7 +136,7 @@ __device__ void build_group_table(const Plan& P, const ShortPlan& SP, double* sc
       }
     }
     double sn, cs;
-    expi_tab(over_hbar(P, th), sct, sn, cs);
+    expi_tab(over_hbar(P, th), B.sct, sn, cs);
     if (kind == GT_POST) sn = -sn;
     if (kind == GT_U || kind == GT_REL) {
       const double h = SP.fscale[gi][0], l = SP.fscale[gi][1];
@@ -148,7 +147,10 @@ __device__ void build_group_table(const Plan& P, const ShortPlan& SP, double* sc
       cs = -cs;
       sn = -sn;
     }
-    if (not_finite(make_double2(cs, sn))) sc[SC_BAD] = 1.0;
+    if (not_finite(make_double2(cs, sn))) {
+      sc[SC_BAD] = 1.0;
+      __stcg(B.bar + BAR_BAD, 1u);
+    }
     __stcg(dst + e, to_mult(make_double2(cs, sn), M61));
   }
 }
@@ -387,6 +389,9 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
   for (int r = team; r < nreg && r < mine; r += TEAMS)
     load_chunk<N>(C, G, psi, blockIdx.x + (int64_t)r * gridDim.x, S.reg + r * S.region_elems, tt, nt, S.s.mbar + r);
 
+  // the launch's last passes have no sum after them that could end it: they ask
+  // whether any CTA noted an entry
+  const bool bad = noted_bad(S.s.sc) || (POST && __ldcg(B.bar + BAR_BAD) != 0);
   int r = team % nreg;
   unsigned use = team / nreg;
   for (int64_t i = team; i < mine; i += TEAMS) {
@@ -475,6 +480,7 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
         Y += d < 32 ? ((unsigned)es[2 * w + 1] >> d) + 1u : 1u;
       }
       bs = block_scale(E, Y, 4, FX_BITS);
+      bs.poison |= bad;
     }
     int eo = bs.eo;
 
@@ -640,6 +646,7 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
     if (g >= 3) acc.merge_rt(2 + l0, accg, 1);
     acc.merge_rt(D, accg, 2);
   }
+  if (MODE != SM_NONE && bad) acc.a[0] = __longlong_as_double(0x7ff8000000000000ll);
   if (MODE != SM_NONE) block_record<double>(B, S.s.red, slot, acc, D + 1);
   __syncthreads();
 }
@@ -690,7 +697,7 @@ __global__ void __launch_bounds__(short64_threads(N), 1)
     centre_after_potential(P, S.s, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
   }
-  build_group_table<N>(P, SP, sc, B.sct, GT_U, SP.tabT);
+  build_group_table<N>(P, SP, B, sc, GT_U, SP.tabT);
   if (!grid_sync(B, &sflag)) return;
 
   for (int64_t u = 0; u < RN.n_units; ++u) {
@@ -717,8 +724,8 @@ __global__ void __launch_bounds__(short64_threads(N), 1)
     centre_after_kinetic(P, S.s, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
     if (hasv) build_v_short(P, SP, B, S.s);
-    build_group_table<N>(P, SP, sc, B.sct, GT_K, SP.tabT);
-    if (final_unit) build_group_table<N>(P, SP, sc, B.sct, GT_POST, SP.tabQ);
+    build_group_table<N>(P, SP, B, sc, GT_K, SP.tabT);
+    if (final_unit) build_group_table<N>(P, SP, B, sc, GT_POST, SP.tabQ);
     if (!grid_sync(B, &sflag)) return;
     if (hasv) load_v64<N>(P, SP, B, S);
     if (threadIdx.x < D) sc[SC_Q + threadIdx.x] = sc[SC_QN + threadIdx.x];
@@ -744,7 +751,7 @@ __global__ void __launch_bounds__(short64_threads(N), 1)
       centre_after_potential(P, S.s, RN.motion);
       if (sc[SC_ERR] != 0.0) goto done;
       if (!final_unit) {
-        build_group_table<N>(P, SP, sc, B.sct, GT_REL, SP.tabT);
+        build_group_table<N>(P, SP, B, sc, GT_REL, SP.tabT);
         if (!grid_sync(B, &sflag)) return;
       }
     }
@@ -758,7 +765,12 @@ done:
       B.ctrl[a] = sc[SC_Q + a];
       B.ctrl[8 + a] = sc[SC_P + a];
     }
-    if (sc[SC_ERR] != 0.0) atomicExch(B.status, (int)sc[SC_ERR]);
+    if (sc[SC_ERR] != 0.0) {
+      atomicExch(B.status, (int)sc[SC_ERR]);
+      // every CTA stopped at the same sum; the one that noted the entry may
+      // have had no chunk to mark
+      if (__ldcg(B.bar + BAR_BAD) != 0) ((double2*)B.psi)[0].x = __longlong_as_double(0x7ff8000000000000ll);
+    }
   }
   if (threadIdx.x == 0 && sc[SC_BAD] != 0.0) atomicExch(B.status, ST_NONFINITE);
 }
