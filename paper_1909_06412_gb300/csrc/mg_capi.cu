@@ -42,6 +42,23 @@ constexpr int RESIDENT_CAP = 96 * 1024;  // bytes per smem region when tiles sta
 constexpr int SHORT64_TABLE = 3 * 4096;  // entries of one group multiplier table of the FP64 short-axis kernel
 constexpr int CHUNK_REGION = 64 * 1024;  // bytes per smem region otherwise
 
+// Lets launches of `fn` use `bytes` of dynamic shared memory.  The limit is one
+// value per kernel function, for all contexts and threads of the process, so it
+// is only ever raised, and at once to all that a CTA can have: whatever another
+// context's launches need stays allowed.
+bool allow_smem(const void* fn, size_t bytes) {
+  cudaFuncAttributes a;
+  int dev = 0, cap = 0;
+  if (cudaFuncGetAttributes(&a, fn) != cudaSuccess) return false;
+  if ((size_t)a.maxDynamicSharedSizeBytes >= bytes) return true;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&cap, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) != cudaSuccess)
+    return false;
+  cap -= (int)a.sharedSizeBytes;
+  return (int)bytes <= cap &&
+         cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, cap) == cudaSuccess;
+}
+
 size_t align256(size_t x) { return (x + 255) & ~size_t(255); }
 
 struct Layout {
@@ -250,7 +267,7 @@ bool plan64(const Plan& P, int sms, Plan& Q) {
   for (int kind = 0; kind < 4; ++kind) {
     void* fn = propagate64_kernel(kind, Q.D);
     int occ = 0;
-    if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, Q.smem_bytes) != cudaSuccess ||
+    if (!allow_smem(fn, Q.smem_bytes) ||
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, Q.smem_bytes) != cudaSuccess || occ < 1) {
       cudaGetLastError();
       return false;
@@ -671,6 +688,7 @@ struct mg_ctx {
   std::vector<double> host;  // staging for psi
   std::vector<double> back;  // mg_get_observables' read-back
   std::vector<double> gam;
+  std::vector<const void*> allowed;  // kernels whose shared memory was asked for (allow_smem)
   double ctrl[32];
 };
 
@@ -702,11 +720,17 @@ mg_status upload_ctrl(mg_ctx* c) {
   return cuda_ok(cudaMemcpyAsync(c->B.ctrl, c->ctrl, 17 * sizeof(double), cudaMemcpyHostToDevice, c->stream));
 }
 
+// allow_smem, asked once per context and kernel: a context launches a kernel
+// with one size, and the limit is never lowered.
+bool allow_smem(mg_ctx* c, const void* fn, size_t bytes) {
+  if (std::find(c->allowed.begin(), c->allowed.end(), fn) != c->allowed.end()) return true;
+  if (!allow_smem(fn, bytes)) return false;
+  c->allowed.push_back(fn);
+  return true;
+}
+
 mg_status launch_plain(mg_ctx* c, void* fn, void** args, size_t smem) {
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return MG_ERR_CUDA;
-  }
+  if (!allow_smem(c, fn, smem)) return MG_ERR_CUDA;
   cudaError_t e = cudaLaunchKernel(fn, dim3(c->P.nblocks), dim3(THREADS), args, smem, c->stream);
   c->launches++;
   return cuda_ok(e);
@@ -866,10 +890,9 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
   tile_plan(P);
   for (int kind = 0; kind < 4; ++kind) {
     void* fn = propagate_kernel(P.prec, kind);
-    if (P.smem_bytes > 48 * 1024)
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes);
     int occ = 0;
-    if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, P.smem_bytes) != cudaSuccess || occ < 1) {
+    if (!allow_smem(fn, P.smem_bytes) ||
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, P.smem_bytes) != cudaSuccess || occ < 1) {
       delete c;
       return MG_ERR_UNSUPPORTED;
     }
@@ -915,7 +938,7 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
     void* fn = P.prec == 0 ? short64_kernel(c->SP.n) : short_kernel(c->SP.n, c->SP.tma, c->SP.tc);
     int occ = 0;
     // the tensor-core variant holds 64 TMEM columns per CTA (512 per SM)
-    if (fn && cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->SP.smem_bytes) == cudaSuccess &&
+    if (fn && allow_smem(fn, c->SP.smem_bytes) &&
         cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, c->SP.threads, c->SP.smem_bytes) == cudaSuccess &&
         occ >= 1 && (!c->SP.tc || occ * 64 <= 512)) {
       c->SP.nblocks = std::min(MAXBLOCKS, occ * sms);
@@ -1190,9 +1213,7 @@ mg_status mg_propagate(mg_ctx* c, int64_t n_steps, double dt, const char* scheme
   Plan& G = general_plan(c);
   void* fn = G.fixed64 ? propagate64_kernel(c->P.pot_kind, c->P.D) : propagate_kernel(c->P.prec, c->P.pot_kind);
   if (!fn) return MG_ERR_UNSUPPORTED;
-  if (G.smem_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, G.smem_bytes) != cudaSuccess)
-    return MG_ERR_CUDA;
+  if (!allow_smem(c, fn, G.smem_bytes)) return MG_ERR_CUDA;
   void* args[] = {&G, &B, &R};
   cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(G.nblocks), dim3(THREADS), args, G.smem_bytes, c->stream);
   c->launches++;
@@ -1215,9 +1236,7 @@ mg_status launch_regrid(mg_ctx* c, const RegridArgs& R) {
   if (s != MG_OK) return s;
   void* fn = regrid_kernel(c->P.prec, c->pot_set ? c->P.pot_kind : MG_POT_HARMONIC);
   if (!fn) return MG_ERR_UNSUPPORTED;
-  if (c->P.smem_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, c->P.smem_bytes) != cudaSuccess)
-    return MG_ERR_CUDA;
+  if (!allow_smem(c, fn, c->P.smem_bytes)) return MG_ERR_CUDA;
   RegridArgs r = R;
   void* args[] = {&c->P, &c->B, &r};
   cudaError_t e = cudaLaunchCooperativeKernel(fn, dim3(c->P.nblocks), dim3(THREADS), args, c->P.smem_bytes, c->stream);
@@ -1399,8 +1418,7 @@ mg_status mg_adjoint(mg_ctx* c, int64_t n_steps, double dt, const char* scheme, 
   const size_t smem = (size_t)P.smem_bytes + 2 * (((size_t)P.region_bytes + 15) & ~size_t(15));
   void* fn = adjoint_kernel(P.pot_kind);
   if (!fn || smem > 227 * 1024) return MG_ERR_UNSUPPORTED;
-  if (cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return MG_ERR_CUDA;
+  if (!allow_smem(fn, smem)) return MG_ERR_CUDA;
   int occ = 0, dev = 0, sms = 0;
   if (cudaGetDevice(&dev) != cudaSuccess || cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
       cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, smem) != cudaSuccess)
@@ -1669,9 +1687,7 @@ extern "C" mg_status mg_propagate_noalloc(int D, const int64_t* N, const double*
   tile_plan(P);
   void* fn = propagate_kernel(P.prec, pot_kind);
   if (!fn) return MG_ERR_UNSUPPORTED;
-  if (P.smem_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes) != cudaSuccess)
-    return MG_ERR_CUDA;
+  if (!allow_smem(fn, P.smem_bytes)) return MG_ERR_CUDA;
   int occ = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&occ, fn, THREADS, P.smem_bytes) != cudaSuccess || occ < 1)
     return MG_ERR_UNSUPPORTED;
@@ -1728,9 +1744,7 @@ extern "C" mg_status mg_propagate_noalloc(int D, const int64_t* N, const double*
 
   // ---- launches: A tables for the starting p-centre, then the propagation ----
   void* targs[] = {&P, &B};
-  if (P.smem_bytes > 48 * 1024 &&
-      cudaFuncSetAttribute(init_tables_kernel(P.prec), cudaFuncAttributeMaxDynamicSharedMemorySize, P.smem_bytes) != cudaSuccess)
-    return MG_ERR_CUDA;
+  if (!allow_smem(init_tables_kernel(P.prec), P.smem_bytes)) return MG_ERR_CUDA;
   if (cudaLaunchKernel(init_tables_kernel(P.prec), dim3(P.nblocks), dim3(THREADS), targs, P.smem_bytes, st) != cudaSuccess)
     return MG_ERR_CUDA;
   Run R;
@@ -1996,7 +2010,7 @@ mg_status mg_batch_create(mg_batch** out, int nprob, mg_ctx* const* ctxs, int cl
   for (int ctas = 1; ctas <= 2; ++ctas) {
     void* f = batch_kernel(prec, ctas);
     int n = 0;
-    if (cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize, A.smem_bytes) != cudaSuccess) {
+    if (!allow_smem(f, A.smem_bytes)) {
       delete b;
       return MG_ERR_CUDA;
     }
