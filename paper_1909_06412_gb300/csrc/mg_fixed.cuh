@@ -15,12 +15,20 @@
 // bounds every intermediate modulus: the first multiplication (|m| <= 1)
 // returns half the product, so 2^61 bounds the norm after it; later ones keep
 // it, and a DFT of n points returns DFT(x) / 2^S: norm factor sqrt(n) / 2^S, at
-// most sqrt(12)/2 for S = 1, and at most twice the norm before the division.
-// Every rounding is to the integer grid and unbiased: a bias, however small
-// beside the rounding noise, is the same vector in every pass over a state
-// that changes little between passes, and adds up over thousands of passes.
-// Ties and halves are decided by low bits of the line's own data (LineBits),
-// products are corrected for the mean of their dropped low parts.
+// most sqrt(12)/2 for S = 1, and at most twice the norm before the division
+// (sqrt(8) times it in idft8_late).
+// Every rounding of the state is to the integer grid and unbiased: a bias,
+// however small beside the rounding noise, is the same vector in every pass over
+// a state that changes little between passes, and adds up over thousands of
+// passes.  The conversion rounds to nearest, ties and halves are decided by low
+// bits of the line's own data (tie_of, LineBits), and products are corrected for
+// the mean of the low parts and bits that they drop.  Only a product of two
+// multipliers (cmul_m) keeps a mean of 2^-60, far below an FP64 table entry's
+// rounding.  Error against 80-bit arithmetic of localised packets on moving
+// grids, the FP64 units' passes -> these: 12^4 2.5e-15 -> 1.4e-15, 16^4 3.2e-15
+// -> 1.0e-15, 8^5 2.2e-15 -> 1.3e-15, 64^3 2.9e-15 -> 2.4e-15, 512 x 384 1.9e-15
+// -> 1.4e-15 (with truncating conversions and uncorrected bits 4.3e-15, 5.4e-15,
+// 5.4e-15, 4.3e-15, 2.0e-15).
 //
 // Multipliers are complex numbers of modulus at most 1 in two 31-bit words
 // per component: value = (h 2^31 + l) / 2^61, 0 <= l < 2^31.
@@ -79,16 +87,20 @@ __host__ __device__ __forceinline__ int madhi(int a, int b, int c) {
 // x * m (HALF: half of it) for a multiplier m, |x| < 2^61 (2^62).  Without
 // LOW the products of the low words are dropped: positive, one unit (half) on
 // average, they cancel in the real part and are added to the imaginary
-// part's half for rounding.
-template <bool HALF, bool LOW> __host__ __device__ __forceinline__ I2 cmul(I2 x, int4 m) {
+// part's half for rounding.  The lowest bits of x are dropped: in a value
+// that comes from to_fixed that is its rounding (odd = 0), elsewhere (odd = -1)
+// it takes one half on average, whose product with m, the same for every x, is
+// added (to the sums of the low products; the imaginary one has to stay below
+// 2^31, hence the 2^30).
+template <bool HALF, bool LOW> __host__ __device__ __forceinline__ I2 cmul(I2 x, int4 m, int odd = 0) {
   constexpr int SH = HALF ? 30 : 29;
   const int rh = m.x, rl = m.y, ih = m.z, il = m.w;
   const int xh = hi32(x.x), xl = lo31(x.x), yh = hi32(x.y), yl = lo31(x.y);
   const int nh = -ih, nl = -il;
-  long long cr = 1LL << (SH - 1), ci = (1LL << (SH - 1)) + (1LL << 30);
+  long long cr = 1LL << (SH - 1), ci = (1LL << (SH - 1)) + (LOW ? 1LL << 31 : 1LL << 30);
   if (LOW) {
-    ci = wide(madhi(xl, il, madhi(yl, rl, 0)), 2, cr);
-    cr = wide(madhi(xl, rl, madhi(yl, nl, 0)), 2, cr);
+    ci = wide(madhi(xl, il, madhi(yl, rl, (((rh + ih) >> 3) & odd) - (1 << 30))), 2, ci);
+    cr = wide(madhi(xl, rl, madhi(yl, nl, ((rh + nh) >> 3) & odd)), 2, cr);
   }
   cr = wide(yl, nh, wide(yh, nl, wide(xl, rh, wide(xh, rl, cr))));
   ci = wide(yl, rh, wide(yh, rl, wide(xl, ih, wide(xh, il, ci))));
@@ -97,7 +109,7 @@ template <bool HALF, bool LOW> __host__ __device__ __forceinline__ I2 cmul(I2 x,
 }
 // a product of multipliers, which need fewer bits
 __host__ __device__ __forceinline__ I2 cmul_m(I2 x, int4 m) { return cmul<false, false>(x, m); }
-__host__ __device__ __forceinline__ I2 cmul_half(I2 x, int4 m) { return cmul<true, true>(x, m); }
+__host__ __device__ __forceinline__ I2 cmul_half(I2 x, int4 m, int odd) { return cmul<true, true>(x, m, odd); }
 
 // The multiplier words of v, scale = 2^61, and of a product held as integers
 // with scale 2^60.
@@ -148,13 +160,14 @@ __host__ __device__ __forceinline__ void idft4(I2& v0, I2& v1, I2& v2, I2& v3, L
   }
 }
 
-// 1 - sqrt(3)/2, 1/(2 sqrt(2)) and 1/(4 sqrt(2)), times 2^63
+// 1 - sqrt(3)/2, 1/(2 sqrt(2)), 1/(4 sqrt(2)) and 1 - 1/sqrt(2), times 2^63
 constexpr int C3H = 575416509, C3L = 516773425;
 // 1 - pi/4 and 1/3, times 2^63 (rotate_turns)
 constexpr int C1MPI4H = 921707869, C1MPI4L = 1867226854;
 constexpr int C13H = 1431655765, C13L = 715827883;
 constexpr int C4H = 1518500249, C4L = 2121767201;
 constexpr int C8H = 759250124, C8L = 2134625425;
+constexpr int C2H = 1257966796, C2L = 51432894;
 
 // three points, unscaled: v0 +- via sqrt(3)/2 d = d - (1 - sqrt(3)/2) d
 template <bool INV> __host__ __device__ __forceinline__ void idft3(I2& v0, I2& v1, I2& v2, LineBits b) {
@@ -191,6 +204,29 @@ template <bool INV, int S> struct IDft<INV, 12, S> {
     for (int r = 0; r < 12; ++r) x[r] = y[r];
   }
 };
+
+// 8 points, divided at the end: half the rounding noise of the form below, for
+// inputs that leave room for the growth of sqrt(8).
+template <bool INV, int S> __host__ __device__ __forceinline__ void idft8_late(I2* x) {
+  const LineBits lb = line_bits(x[0], x[1]);
+  I2 a[4], b[4];
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    a[r] = iadd(x[r], x[r + 4]);
+    b[r] = isub(x[r], x[r + 4]);
+  }
+  const I2 s1 = iadd(b[1], imul_si<INV>(b[1])), s3 = isub(imul_si<INV>(b[3]), b[3]);
+  b[1] = I2{s1.x - mul_c(s1.x, C2H, C2L), s1.y - mul_c(s1.y, C2H, C2L)};
+  b[3] = I2{s3.x - mul_c(s3.x, C2H, C2L), s3.y - mul_c(s3.y, C2H, C2L)};
+  b[2] = imul_si<INV>(b[2]);
+  idft4<INV, S>(a[0], a[1], a[2], a[3], lb);
+  idft4<INV, S>(b[0], b[1], b[2], b[3], lb);
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    x[2 * r] = a[r];
+    x[2 * r + 1] = b[r];
+  }
+}
 
 // 8 by one decimation-in-frequency split.  The shift follows the first
 // butterflies; the 1/sqrt(2) rotations carry it in their constant.
@@ -296,8 +332,7 @@ __host__ __device__ __forceinline__ int fx_exponent(unsigned m) {
   return e < FX_EMIN ? FX_EMIN : e;
 }
 __host__ __device__ __forceinline__ unsigned fx_square(unsigned m, int emax) {
-  const int e = (int)(m >> 20);
-  if (e < FX_EMIN) return 257u * 257u;
+  const int e = fx_exponent(m);  // an empty or next to empty group adds a unit
   const unsigned a = ((m >> 12) & 0xffu) + 257u;  // 1.mantissa 2^8, rounded up
   const int d = 2 * (emax - e);
   return d < 20 ? ((a * a) >> d) + 1u : 1u;
@@ -308,6 +343,7 @@ struct BlockScale {
   int ref;     // see to_fixed
   int eo;      // value = integer * 2^eo
   int poison;  // an infinity or NaN is in the block
+  int spare;   // the norm is below 2^(bits - spare / 2)
 };
 // From the largest exponent field E and the sum Y of the groups' squares
 // relative to it (each group of `vals` values): norm < 2^(E - 1031 + half).
@@ -324,23 +360,31 @@ __host__ __device__ __forceinline__ BlockScale block_scale(int E, unsigned Y, in
   s.ref = 54 - bits + E + half;
   s.eo = E - 1031 + half - bits;
   s.poison = E >= 2047;
+  s.spare = lg & 1;
   return s;
 }
 
-// FP64 value (as its two words) to an even integer at the block's scale (the
-// multiplications drop the lowest bit).  Truncated towards zero; the values
-// near a block's largest, which make up its norm, are exact.
-__host__ __device__ __forceinline__ long long to_fixed(int hi, unsigned lo, int ref) {
+// FP64 value (as its two words) to an integer at the block's scale whose lowest
+// bit is to be dropped, as the multiplications do: that leaves the nearest even
+// integer.  A tie goes away from zero for tie = 0, towards it for tie = 1
+// (tie_of: by a low bit of the line's data); the ten spare bits below the
+// mantissa keep everything else from being moved by it.  The mean error is zero:
+// cut off towards zero, it would be a vector that is the same in every pass, and
+// add up.
+__host__ __device__ __forceinline__ long long to_fixed(int hi, unsigned lo, int ref, int tie) {
   const unsigned mh = ((unsigned)hi & 0xfffffu) | 0x100000u;
-  const unsigned long long m = (((unsigned long long)mh << 32) | lo) << 10;
+  const long long m = (long long)((((unsigned long long)mh << 32) | lo) << 10);
   // above 63 the value is zero; below zero only for a value above the bound
   // (an infinity or NaN as a multiplier, which its reader notes: SC_BAD)
   unsigned sh = (unsigned)(ref - (int)(((unsigned)hi >> 20) & 0x7ffu));
   sh = sh > 63u ? 63u : sh;
-  const unsigned long long v = (m >> sh) & ~1ull;
   const long long s = (long long)(hi >> 31);
-  return ((long long)v ^ s) - s;
+  return (((m - tie) ^ s) >> sh) + 1;
 }
+__host__ __device__ __forceinline__ I2 to_fixed(I2 v, int ref, int tie) {
+  return I2{to_fixed(hi32(v.x), (unsigned)v.x, ref, tie), to_fixed(hi32(v.y), (unsigned)v.y, ref, tie)};
+}
+__host__ __device__ __forceinline__ int tie_of(I2 a, I2 b) { return (int)(((unsigned)a.x ^ (unsigned)b.y) & 1u); }
 #ifdef __CUDACC__
 // An infinity or NaN, which multiplier words cannot carry: where a phase
 // overflows its table entries are NaN.  Whoever turns such an entry into words
@@ -353,10 +397,6 @@ constexpr int BAR_BAD = 32;
 __device__ __forceinline__ bool noted_bad(const double* sc) { return __double2hiint(sc[SC_BAD]) != 0; }
 __device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
 __device__ __forceinline__ bool not_finite(double2 v) { return not_finite(v.x) || not_finite(v.y); }
-__device__ __forceinline__ I2 to_fixed2(double2 v, int ref) {
-  return I2{to_fixed(__double2hiint(v.x), (unsigned)__double2loint(v.x), ref),
-            to_fixed(__double2hiint(v.y), (unsigned)__double2loint(v.y), ref)};
-}
 // integer * 2^eo: converted by the FP64 unit (rounded to nearest), then the
 // exponent field is moved; zero stays zero.
 __device__ __forceinline__ double from_fixed(long long v, int eo) {

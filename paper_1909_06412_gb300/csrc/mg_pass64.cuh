@@ -24,14 +24,14 @@ namespace mgk {
 namespace {
 
 constexpr double INV_2PI = 0.15915494309189535, INV_2PI_LO = -9.839338337591243e-18;
-constexpr int PASS_BITS = 60;  // norm bound of a chunk; growth within a transform at most sqrt(2)
+constexpr int PASS_BITS = 61;  // norm bound of a chunk, also after every pass of its transform
 
 extern __shared__ __align__(16) unsigned char smem_raw64[];
 
 // Multiplier words of v 2^s, |v| 2^s <= 1, by integer operations.
 __device__ __forceinline__ int4 mult_bits(double2 v, int s) {
-  const long long a = to_fixed(__double2hiint(v.x), (unsigned)__double2loint(v.x), 1024 - s);
-  const long long b = to_fixed(__double2hiint(v.y), (unsigned)__double2loint(v.y), 1024 - s);
+  const long long a = to_fixed(__double2hiint(v.x), (unsigned)__double2loint(v.x), 1024 - s, 0) & ~1ll;
+  const long long b = to_fixed(__double2hiint(v.y), (unsigned)__double2loint(v.y), 1024 - s, 0) & ~1ll;
   return make_int4((int)(a >> 31), (int)(a & 0x7fffffff), (int)(b >> 31), (int)(b & 0x7fffffff));
 }
 // floor(log2 n): conj(A)/n is held times 2^this
@@ -91,7 +91,7 @@ __device__ __forceinline__ double turns_scale(double x, double* sc) {
 // 64-bit fraction (exact); its first two bytes select table factors, the rest
 // is a series: a = 2 pi f / 2^16, |f| <= 1/2, sin = a - a^3/6, cos = 1 - a^2/2
 // (the next terms are below 2^-61).
-__device__ __forceinline__ I2 rotate_turns(I2 x, double t, float eps, const int4* tab) {
+__device__ __forceinline__ I2 rotate_turns(I2 x, double t, float eps, const int4* tab, int odd) {
   const int hi = __double2hiint(t);
   const unsigned long long m =
       ((unsigned long long)(((unsigned)hi & 0xfffffu) | 0x100000u) << 32) | (unsigned)__double2loint(t);
@@ -118,7 +118,7 @@ __device__ __forceinline__ I2 rotate_turns(I2 x, double t, float eps, const int4
   const long long s3 = wide(c2h, e3, 0) >> 29;         // a^3 / 2, times 2^61
   const long long sn = es - mul_c(s3, C13H, C13L);
   const int4 w = make_int4((int)(cs >> 31), (int)(cs & 0x7fffffff), (int)(sn >> 31), (int)(sn & 0x7fffffff));
-  return cmul<false, true>(cmul<false, true>(cmul<false, true>(x, t1), t2), w);
+  return cmul<false, true>(cmul<false, true>(cmul<false, true>(x, t1, odd), t2, -1), w, -1);
 }
 
 // One Stockham pass of radix R over L lines of length n (see stockham_pass),
@@ -161,12 +161,12 @@ __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* _
           w.z = -w.z;
           w.w = -w.w;
         }
-        v[r] = cmul<false, true>(v[r], w);
+        v[r] = cmul<false, true>(v[r], w, -1);
       }
     } else {
+      const int tie = tie_of(v[0], v[1]);
 #pragma unroll
-      for (int r = 0; r < R; ++r)
-        v[r] = I2{to_fixed(hi32(v[r].x), (unsigned)v[r].x, ref), to_fixed(hi32(v[r].y), (unsigned)v[r].y, ref)};
+      for (int r = 0; r < R; ++r) v[r] = to_fixed(v[r], ref, tie);
       if (pre) {
 #pragma unroll
         for (int r = 0; r < R; ++r) v[r] = cmul<false, true>(v[r], pre[j + r * nR]);
@@ -177,11 +177,14 @@ __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* _
           if (not_finite(m)) *bad = 1.0;
           v[r] = cmul<false, true>(v[r], mult_bits(m, 0));
         }
+      } else {
+#pragma unroll
+        for (int r = 0; r < R; ++r) v[r] = I2{v[r].x & ~1ll, v[r].y & ~1ll};
       }
     }
     const LineBits lb = line_bits(v[0], v[1]);
     if constexpr (R == 8) {
-      IDft<INV, 8, SC>::run(v);
+      idft8_late<INV, SC>(v);
     } else if constexpr (R == 4) {
       idft4<INV, SC>(v[0], v[1], v[2], v[3], lb);
     } else if constexpr (R == 3) {
@@ -204,19 +207,21 @@ __device__ __forceinline__ void stockham64_pass(const I2* __restrict__ in, I2* _
 }
 
 // Transform of L lines; returns the buffer with the result and adds the
-// divisions to eo.  The norm factor of the passes so far is 2^(h/2), h 0 or 1
-// (radix 2, 4, 8: sqrt(R); radix 3 counted as 2).
+// divisions to eo.  The norm is below 2^(PASS_BITS + h/2), h 0 or -1: a pass
+// multiplies it by sqrt(R) (radix 3 counted as 2) and divides by as little as
+// keeps it there.
 template <bool INV>
 __device__ I2* stockham64(I2* in, I2* out, int L, const AxisPlan& ax, const int4* tw, const int4* pre,
-                          const double2* preg, int wsh, int ref, double* bad, int& eo) {
-  int Ns = 1, h = 0;
+                          const double2* preg, int wsh, BlockScale bs, double* bad, int& eo) {
+  const int ref = bs.ref;
+  int Ns = 1, h = -bs.spare;
   const int n = ax.n;
   const Div16 divL((unsigned)L);
   for (int pi = 0; pi < ax.nrad; ++pi) {
     const int R = ax.rad[pi];
     h += R == 8 ? 3 : (R == 2 ? 1 : 2);
-    const int sc = h >> 1;
-    h &= 1;
+    const int sc = (h + 1) >> 1;
+    h -= 2 * sc;
     eo += sc;
     if (R == 8) {
       if (sc == 1) stockham64_pass<INV, 8, 1>(in, out, n, L, divL, Ns, tw, pre, preg, wsh, ref, bad);
@@ -392,10 +397,11 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
     int eo = bs.eo;
     I2* ic = (I2*)cur;
     if (A.fft) {
-      ic = stockham64<INV>(ic, (I2*)oth, nt * W, ax, tw, pre, preg, wsh, bs.ref, S.sc + SC_BAD, eo);
+      ic = stockham64<INV>(ic, (I2*)oth, nt * W, ax, tw, pre, preg, wsh, bs, S.sc + SC_BAD, eo);
       cur = (V*)ic;
     }
     if (postT) eo -= post_shift(n);
+    const int odd = A.fft ? -1 : 0;
     const bool poison = bs.poison || noted_bad(S.sc);
 
     // epilogue: element e of the chunk is tile ti, point j, line w
@@ -405,7 +411,7 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
       const int w = contig ? (int)divn((unsigned)rem) : rem & (W - 1);
       const int j = contig ? rem - w * n : rem >> wsh;
       I2 x = ic[e];
-      if (!A.fft) x = I2{to_fixed(hi32(x.x), (unsigned)x.x, bs.ref), to_fixed(hi32(x.y), (unsigned)x.y, bs.ref)};
+      if (!A.fft) x = to_fixed(x, bs.ref, tie_of(x, x));
       bool nan = poison;
       if (postT) {
         int4 m;
@@ -419,7 +425,7 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
         } else {
           m = ((const int4*)postT)[j];
         }
-        x = cmul<false, true>(x, m);
+        x = cmul<false, true>(x, m, odd);
       }
       V v;
       if (A.red != RED_NONE) {
@@ -438,14 +444,14 @@ __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const Pass
           if (P.minv_general) {
             // the non-separable part of the kinetic phase (see axis_pass)
             const double th = over_hbar(P, -S.sc[SC_TAU] * kinetic_cross<DM>(P, S.tc, S.sc, idx));
-            v = from_fixed2(rotate_turns(x, th * INV_2PI, KIN_TEPS, tab), eo);
+            v = from_fixed2(rotate_turns(x, th * INV_2PI, KIN_TEPS, tab, odd), eo);
             nan = nan || not_finite(th);
           }
         } else {  // RED_V
           double th, g[DM];
           vpoint<KIND, DM>(P, S.tv, idx, sgh, th, g);
           // |x|^2 is the same before and after the phase
-          v = from_fixed2(rotate_turns(x, th, teps, tab), eo);
+          v = from_fixed2(rotate_turns(x, th, teps, tab, odd), eo);
           // an overflowing potential leaves no phase: a NaN, as its sine would be
           nan = nan || not_finite(th);
           const double w2 = nan ? __longlong_as_double(0x7ff8000000000000ll) : fma(v.x, v.x, v.y * v.y);

@@ -22,7 +22,8 @@
 // i + nreg into its region, on an mbarrier that the team taking that chunk
 // waits on.
 //
-// Reductions.  |x|^2 of the integers is summed exactly along a line (the
+// Reductions.  |x|^2 of the integers is summed along a line as integers (each
+// component to 2^-57 or 2^-54 of the chunk's norm, without a mean error; the
 // squares' high and middle parts in two 64-bit sums, the sums weighted by the
 // line's coordinate from running sums of those), and one FP64 value per line
 // and moment is formed at the end of the line.
@@ -328,13 +329,18 @@ __device__ __forceinline__ void store_chunk(const CopyPlan& C, const GroupPlan& 
 
 // Integer sums of |x|^2 along a line, and of |x|^2 times the running count
 // (twice for W = 2): S_k = sum of S_(k-1).  x is cut into its high word (after
-// dropping S bits) and the next B bits: |x|^2 = 2^(64 + 2 S) (H + C 2^(1-B)).
-// S and B are as large as the weighted sums of 16 points leave room for.
+// dropping S bits) and the next B bits, the last of them set: the middle of the
+// interval that B - 1 bits leave, so that the values are not low on average.
+// |x|^2 = 2^(64 + 2 S) (H + C 2^(1-B)).  The sums are exact modulo 2^64; what
+// is taken from them fits: with norm^2 < 2^124.8 (kinetic) or 2^124 the sum of
+// the squared high words is below 2^(60.8 - 2 S) or 2^(60 - 2 S), and a weighted
+// C below 2^B times its root times that of the sum of the squared weights: 2^62.5
+// and 2^61.3 for 12 points, 2^61.7 and 2^61.4 for 16 (norm^2 < 2^122).
 template <int W, int S, int B> struct LineSums {
   unsigned long long h0 = 0, h1 = 0, h2 = 0;
   unsigned long long c0 = 0, c1 = 0, c2 = 0;
   static __device__ __forceinline__ int mid(long long v) {
-    return (int)(__funnelshift_r((unsigned)v, (unsigned)hi32(v), 32 - B + S) & ((1u << B) - 1));
+    return (int)((__funnelshift_r((unsigned)v, (unsigned)hi32(v), 32 - B + S) & ((1u << B) - 1)) | 1u);
   }
   __device__ __forceinline__ void add(I2 v) {
     const int xh = hi32(v.x) >> S, yh = hi32(v.y) >> S, xm = mid(v.x), ym = mid(v.y);
@@ -515,11 +521,12 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
         }
         if (kk == 0) {
           const int4* mt = tabT + row;
+          const int tie = tie_of(x[0], x[N / 2]);
 #pragma unroll
           for (int q = 0; q < N; ++q) {
-            x[q] = I2{to_fixed(hi32(x[q].x), (unsigned)x[q].x, bs.ref), to_fixed(hi32(x[q].y), (unsigned)x[q].y, bs.ref)};
+            x[q] = to_fixed(x[q], bs.ref, tie);
             if (MODE != SM_VONLY) {
-              x[q] = cmul_half(x[q], __ldcg(mt));
+              x[q] = cmul_half(x[q], __ldcg(mt), 0);
               mt += nlo;
             }
           }
@@ -535,7 +542,7 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
             const int4* mt = tabQ + row;
 #pragma unroll
             for (int q = 0; q < N; ++q) {
-              x[q] = cmul_half(x[q], __ldcg(mt));
+              x[q] = cmul_half(x[q], __ldcg(mt), -1);
               mt += nlo;
             }
           }
@@ -553,7 +560,7 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
         if (MODE == SM_KIN) {
           // kinetic moments; the line runs along axis 0 (k = 0, l0 = 0)
           constexpr int SH = 1;
-          LineSums<1, SH, 28> m;
+          LineSums<1, SH, 29> m;
 #pragma unroll
           for (int q = 0; q < N; ++q) m.add(x[q]);
           const double s = moment_scale(eo + SH, bs.poison);
@@ -573,7 +580,7 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
           // potential substep on the line along the last axis: moments, then
           // the phase lf * (last pair's factor at r)
           constexpr int SH = 2;
-          LineSums<2, SH, 26> m;
+          LineSums<2, SH, 27> m;
 #pragma unroll
           for (int q = 0; q < N; ++q) m.add(x[q]);
           const double s = moment_scale(eo + SH, bs.poison);
@@ -607,7 +614,8 @@ __device__ __noinline__ void pass64(const Plan& P, const ShortPlan& SP, const Bu
           lf = cmul_m(lf, S.Gh[hi]);
           const int4* prow = S.Pt + ((D - 2) * N + jm) * (N + 1);
 #pragma unroll
-          for (int q = 0; q < N; ++q) x[q] = cmul<!POST, true>(x[q], to_mult60(cmul_m(lf, prow[q])));
+          for (int q = 0; q < N; ++q)
+            x[q] = cmul<!POST, true>(x[q], to_mult60(cmul_m(lf, prow[q])), MODE == SM_VONLY ? 0 : -1);
           if (!POST) eout += 1;
         }
         {
