@@ -221,7 +221,7 @@ done:
 // registers each is slower by itself.  512 uneven 2D and 3D grids, FP32, two
 // suzuki4 steps: 51.6 ms with one CTA of up to 255 registers a thread, 34.5 ms
 // with two of 128 (spills of about 1 KB a thread); a batch of a few
-// problems per team is 5-8% faster with one (the host's rule, mg_batch_create).
+// problems per team is 5-8% faster with one (the host's rule, mg_rules.h).
 template <typename T, int CTAS>
 __global__ void __launch_bounds__(THREADS, CTAS) k_batch(const __grid_constant__ BatchArgs BA) {
   using V = typename VT<T>::v;

@@ -13,6 +13,7 @@
 
 #include "mg_plan.h"
 #include "mg_regrid.h"
+#include "mg_rules.h"
 #include "mg_short.h"
 #include "mgrid.h"
 
@@ -2000,30 +2001,29 @@ mg_status mg_batch_create(mg_batch** out, int nprob, mg_ctx* const* ctxs, int cl
   cfg.dynamicSmemBytes = A.smem_bytes;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
-  // The kernel that runs two CTAs per SM (where the shared memory of two fits)
-  // from four problems per team on.  With fewer the longest problem decides,
-  // and each team is slower with half the registers: measured on uneven
-  // batches, FP32, against one CTA per SM, 512 problems for 76 teams 1.51x as
-  // fast, 187 problems 0.95x, 51 problems 0.92x; FP64, 368 problems 1.06x.
-  void* fn = nullptr;
-  int ncl = 0;
-  for (int ctas = 1; ctas <= 2; ++ctas) {
+  // teams that the kernel of `ctas` CTAs per SM can run; 0 if it cannot
+  auto teams = [&](int ctas) {
     void* f = batch_kernel(prec, ctas);
     int n = 0;
-    if (!allow_smem(f, A.smem_bytes)) {
-      delete b;
-      return MG_ERR_CUDA;
+    if (!allow_smem(f, A.smem_bytes) || cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess) {
+      cudaGetLastError();
+      return 0;
     }
-    if (cudaOccupancyMaxActiveClusters(&n, f, &cfg) != cudaSuccess || n < 1) {
-      delete b;
-      return MG_ERR_UNSUPPORTED;
-    }
-    if (n > ncl) {
-      fn = f;
-      ncl = n;
-    }
-    if (nprob <= 4 * ncl) break;
+    return n;
+  };
+  if (!allow_smem(batch_kernel(prec, 1), A.smem_bytes)) {
+    delete b;
+    return MG_ERR_CUDA;
   }
+  const int teams1 = teams(1);
+  if (teams1 < 1) {
+    delete b;
+    return MG_ERR_UNSUPPORTED;
+  }
+  const int teams2 = batch_wants_two(nprob, teams1) ? teams(2) : 0;
+  const int ctas = batch_ctas(nprob, teams1, teams2);
+  void* fn = batch_kernel(prec, ctas);
+  const int ncl = ctas == 2 ? teams2 : teams1;
   b->nteams = std::min(std::min(ncl, nprob), MAXTEAMS);
   A.nteams = b->nteams;
 

@@ -1,0 +1,28 @@
+// Host rules of the dispatch that need no device: which variant serves a call,
+// from sizes and counts alone.
+#pragma once
+#include <stdint.h>
+
+namespace mgk {
+
+// The kernel that runs two CTAs per SM (where the shared memory of two fits)
+// pays from four problems per team on: with fewer the longest problem decides,
+// and each team is slower with half the registers.  Measured on uneven 2D and 3D
+// batches, FP32, one CTA per SM against two at p problems per team: teams of two
+// CTAs p = 2.0 0.85x, 2.6 0.87x, 3.2 0.96x, 3.7 0.99x, 4.2 1.25x, 4.7 1.45x, 6.0
+// 1.37x (only 3D grids 2.0 0.96x, 3.2 1.40x, 4.2 1.54x); teams of one 2.0 0.85x,
+// 3.0 0.91x, 3.9 1.01x, 5.0 1.22x; of four 2.6 0.87x, 3.9 1.14x, 5.3 1.54x.  In
+// FP64 the shared memory of two fits for few batches (368 problems of one: 1.06x).
+constexpr int BATCH_TWO_CTAS = 4;
+
+// Whether the two-CTA kernel is worth asking for, with `teams1` teams of the
+// one-CTA kernel.
+inline bool batch_wants_two(int nprob, int teams1) { return nprob > BATCH_TWO_CTAS * teams1; }
+
+// CTAs per SM of the batched kernel: `teams2` teams could run of the two-CTA
+// kernel (0: none, or the question failed).
+inline int batch_ctas(int nprob, int teams1, int teams2) {
+  return batch_wants_two(nprob, teams1) && teams2 > teams1 ? 2 : 1;
+}
+
+}  // namespace mgk

@@ -1,0 +1,32 @@
+"""The host rules of csrc/mg_rules.h, compiled for the host: which kernel variant
+a call gets, from sizes and counts alone."""
+import os
+import shutil
+import subprocess
+
+import pytest
+
+ROOT = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+
+
+@pytest.fixture
+def rule(tmp_path):
+    gxx = shutil.which("g++")
+    if not gxx:
+        pytest.skip("no host compiler")
+
+    def call(*exprs):
+        src, exe = tmp_path / "rules.cpp", tmp_path / "rules"
+        body = "".join(f'  printf("%g\\n", (double)({e}));\n' for e in exprs)
+        src.write_text('#include <cstdio>\n#include "mg_rules.h"\nusing namespace mgk;\nint main() {\n' + body + "}\n")
+        subprocess.run([gxx, "-std=c++17", f"-I{ROOT}/paper_1909_06412_gb300/csrc", "-o", str(exe), str(src)], check=True)
+        return [float(x) for x in subprocess.run([str(exe)], check=True, capture_output=True, text=True).stdout.split()]
+
+    return call
+
+
+def test_batches_fall_back_to_one_cta_per_sm(rule):
+    # two CTAs per SM from four problems per team on, where they are to be had
+    assert rule("batch_ctas(304, 76, 152)", "batch_ctas(305, 76, 152)", "batch_ctas(1, 76, 152)") == [1, 2, 1]
+    # a kernel that cannot run, or runs no more teams, leaves the other one
+    assert rule("batch_ctas(512, 76, 0)", "batch_ctas(512, 76, 76)", "batch_ctas(512, 76, -1)") == [1, 1, 1]
