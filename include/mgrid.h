@@ -250,7 +250,8 @@ int mg_scheme_coefficients(const char* scheme, double* gamma, int max);
  * number of groups, 0 if the grid does not take the short-axis kernel, -1 for
  * an invalid grid.  first_axis and naxes: caller arrays of 8 ints (or NULL);
  * threads, smem_bytes (or NULL): the CTA size and the dynamic shared memory
- * of the cp.async layout (the TMA layout, chosen at mg_create, may differ). */
+ * of the cp.async layout (the TMA layout, chosen at mg_create, may differ).
+ * The FP64 chunk size depends on the number of SMs; the query takes 152. */
 int mg_short_axis_plan(int D, const int64_t* N, int precision, int* first_axis, int* naxes, int* threads,
                        int* smem_bytes);
 

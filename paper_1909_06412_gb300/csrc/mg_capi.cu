@@ -397,21 +397,17 @@ bool short_plan_lpc(const Plan& P, ShortPlan& SP, int tc, int lpc) {
 }
 
 // The plan with the chunk size that suits the grid (FP32 chunks have one size).
-// A pass is bound by latency, not by throughput: measured, a warp takes about
-// 4000 cycles for its lines of one axis whether it shares its scheduler with
-// none or two others, a chunk about 8000 for its copies and waits, and 3000
-// stand for the barrier of a pass.  So a grid with fewer chunks than teams
-// (two per SM) gains from smaller chunks, even at more passes, and a large one
-// keeps the largest.  Microseconds per kinetic unit with the largest chunks
+// A pass is bound by latency (short_pass_cost), so a grid with fewer chunks than
+// teams gains from smaller chunks, even at more passes, and a large one keeps
+// the largest.  Microseconds per kinetic unit with the largest chunks
 // and with the ones chosen: 12^4 126 (288 lines) -> 96 (144); 12^5 137 (288) ->
 // 106 (144); 16^4 137 (256) -> 100 (32); 8^4 94 (256) -> 74 (64); 12^3 69 -> 66;
 // 16^5 and larger keep theirs.
-bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
+bool short_plan(const Plan& P, int sms, ShortPlan& SP, int tc = 0) {
   const int n = short_shape(P.D, P.N);
   if (!n) return false;
   const int full = short_lpc_for(P.prec, n, tc);
   if (P.prec != 0) return short_plan_lpc(P, SP, tc, full);
-  constexpr int64_t TEAMS_ALL = 2 * 152;
   double best = 0;
   bool ok = false;
   for (int d = 1; full / d >= n; ++d) {
@@ -420,9 +416,7 @@ bool short_plan(const Plan& P, ShortPlan& SP, int tc = 0) {
     double cost = 0;
     for (int i = 0; i < C.ngroups; ++i) {
       const GroupPlan& G = C.grp[i];
-      const int64_t waves = (G.nchunks + TEAMS_ALL - 1) / TEAMS_ALL;
-      const int lines = full / d, team = C.threads / 2, rounds = (lines + team - 1) / team;
-      cost += (double)waves * (4.0 * G.g * rounds + 8.0) + 3.0;
+      cost += short_pass_cost(G.nchunks, G.g, full / d, C.threads, sms);
     }
     if (!ok || cost < best) {
       best = cost;
@@ -933,7 +927,7 @@ mg_status mg_create_ex(mg_ctx** out, int D, const int64_t* N, const double* dq, 
   }
 
   // short-axis kernel: one CTA per SM, all co-resident
-  if (!(flags & MG_CREATE_GENERAL_KERNEL) && short_plan(P, c->SP, want_tc)) {
+  if (!(flags & MG_CREATE_GENERAL_KERNEL) && short_plan(P, sms, c->SP, want_tc)) {
     c->SP.tma = !(flags & MG_CREATE_NO_TMA) && short_tma_maps(P, c->SP, d_psi) ? 1 : 0;
     if (c->SP.tma && !short_tma_smem(P, c->SP)) c->SP.tma = 0;
     void* fn = P.prec == 0 ? short64_kernel(c->SP.n) : short_kernel(c->SP.n, c->SP.tma, c->SP.tc);
@@ -1514,7 +1508,7 @@ int mg_short_axis_plan(int D, const int64_t* N, int precision, int* first_axis, 
     P.maxn = std::max(P.maxn, P.ax[l].n);
   }
   ShortPlan SP;
-  if (!short_plan(P, SP)) return 0;
+  if (!short_plan(P, 152, SP)) return 0;
   for (int g = 0; g < SP.ngroups; ++g) {
     if (first_axis) first_axis[g] = SP.grp[g].l0;
     if (naxes) naxes[g] = SP.grp[g].g;

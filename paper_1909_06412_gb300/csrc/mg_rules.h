@@ -25,4 +25,16 @@ inline int batch_ctas(int nprob, int teams1, int teams2) {
   return batch_wants_two(nprob, teams1) && teams2 > teams1 ? 2 : 1;
 }
 
+// Cost of the passes of the FP64 short-axis kernel over one group of g axes, for
+// `nchunks` chunks of `lines` lines on `sms` SMs, in thousands of cycles.  A pass
+// is bound by latency, not by throughput: measured, a warp takes about 4000
+// cycles for its lines of one axis whether it shares its scheduler with none or
+// two others, a chunk about 8000 for its copies and waits, and 3000 stand for the
+// barrier of a pass.  Chunks are dealt to two teams per SM.
+inline double short_pass_cost(int64_t nchunks, int g, int lines, int threads, int sms) {
+  const int64_t teams = 2 * (int64_t)sms, waves = (nchunks + teams - 1) / teams;
+  const int team = threads / 2, rounds = (lines + team - 1) / team;
+  return (double)waves * (4.0 * g * rounds + 8.0) + 3.0;
+}
+
 }  // namespace mgk

@@ -30,3 +30,10 @@ def test_batches_fall_back_to_one_cta_per_sm(rule):
     assert rule("batch_ctas(304, 76, 152)", "batch_ctas(305, 76, 152)", "batch_ctas(1, 76, 152)") == [1, 2, 1]
     # a kernel that cannot run, or runs no more teams, leaves the other one
     assert rule("batch_ctas(512, 76, 0)", "batch_ctas(512, 76, 76)", "batch_ctas(512, 76, -1)") == [1, 1, 1]
+
+
+def test_chunk_costs_follow_the_number_of_sms(rule):
+    # 200 chunks are one wave for the 304 teams of 152 SMs, two for those of 76
+    one, two, more = rule("short_pass_cost(200, 3, 144, 384, 152)", "short_pass_cost(200, 3, 144, 384, 76)",
+                          "short_pass_cost(400, 3, 144, 384, 152)")
+    assert one < two == more
