@@ -252,14 +252,9 @@ void tile_plan(Plan& P) {
 }
 
 // Plan of k_propagate64 in place of P's kernel, for FP64 grids with enough
-// points.  The integer passes have the higher throughput and the longer
-// latency for a few points (one CTA per SM either way): measured per yoshida4
-// call 1.39x on 128^3 (13,800 points per SM) and 1.17x on 128 x 2048 (1725),
-// 0.89x on 256^2 (431) and 0.80x on 32^3 (216); the line is drawn between.
-constexpr int64_t FIXED64_POINTS = 1024;  // per SM
-
+// points (integer_passes; one CTA per SM either way).
 bool plan64(const Plan& P, int sms, Plan& Q) {
-  if (P.prec != 0 || P.npts < FIXED64_POINTS * sms) return false;
+  if (P.prec != 0 || !integer_passes(P.D, P.npts, sms)) return false;
   Q = P;
   Q.fixed64 = 1;
   Q.nblocks = sms;

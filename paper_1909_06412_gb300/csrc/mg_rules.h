@@ -25,6 +25,23 @@ inline int batch_ctas(int nprob, int teams1, int teams2) {
   return batch_wants_two(nprob, teams1) && teams2 > teams1 ? 2 : 1;
 }
 
+// Whether the general kernel's FP64 passes run on the integer units
+// (mg_pass64.cuh).  They have the higher throughput and the longer latency for a
+// few points; a grid of more axes has more passes with less work in each.  FP64
+// units against integer units, yoshida4 calls, by points per SM: two axes 431
+// 0.89x, 1035 1.26-1.29x, 1091 1.14-1.15x, 1724 1.27x; three 216 0.80x, 1035
+// 1.13-1.16x, 1091 1.03-1.05x, 13,800 1.36x; four 1227 0.98x, 1381 1.04-1.06x,
+// 2182 1.05x, 11,050 1.23x; five 1091 0.93x, 2182 1.01x, 2910 0.99x, 12,431
+// 1.05x; axes of 12.8 points on average and six of them 29,466 1.09x, but of 8.7
+// (six) 2910 0.98x, of 7.7 (seven) 10,347 0.97x, of 6.9 (eight) 34,923 0.90x.
+inline bool integer_passes(int D, int64_t npts, int sms) {
+  const int64_t per_sm = D <= 3 ? 1024 : 1024 * (int64_t)D / 3;
+  if (npts < per_sm * sms) return false;
+  int64_t n9 = 1;
+  for (int l = 0; l < D; ++l) n9 *= 9;
+  return D <= 3 || npts >= n9;  // nine points an axis on average
+}
+
 // Cost of the passes of the FP64 short-axis kernel over one group of g axes, for
 // `nchunks` chunks of `lines` lines on `sms` SMs, in thousands of cycles.  A pass
 // is bound by latency, not by throughput: measured, a warp takes about 4000

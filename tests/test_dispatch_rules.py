@@ -37,3 +37,11 @@ def test_chunk_costs_follow_the_number_of_sms(rule):
     one, two, more = rule("short_pass_cost(200, 3, 144, 384, 152)", "short_pass_cost(200, 3, 144, 384, 76)",
                           "short_pass_cost(400, 3, 144, 384, 152)")
     assert one < two == more
+
+
+def test_grids_of_many_short_axes_keep_the_fp64_units(rule):
+    grids = {(54, 54, 54): 1, (32, 32, 32): 0, (162, 972): 1, (256, 256): 0, (24,) * 4: 1, (18, 18, 24, 24): 0,
+             (12, 12, 12, 12, 18): 1, (8, 12, 8, 18, 12): 0, (12, 12, 12, 12, 12, 18): 1, (6, 8, 6, 8, 6, 12): 0,
+             (6, 8, 8, 12, 8, 12): 0, (8,) * 6 + (6,): 0, (4,) * 7 + (12,): 0, (6, 6, 6, 6, 8, 8, 8, 8): 0}
+    size = {N: "*".join(f"{n}ll" for n in N) for N in grids}
+    assert rule(*(f"integer_passes({len(N)}, {size[N]}, 152)" for N in grids)) == list(grids.values())
