@@ -348,7 +348,9 @@ template <typename V> struct Smem {
   size_t end;   // bytes used
 };
 
-template <typename V> __device__ Smem<V> carve(const Plan& P, const Bufs& B, unsigned char* base) {
+// F64: a plan of k_propagate64 (Plan::fixed64), whose sincos table is twice as
+// large.  A constant, so that the offsets behind it cost no registers elsewhere.
+template <typename V, bool F64 = false> __device__ Smem<V> carve(const Plan& P, const Bufs& B, unsigned char* base) {
   Smem<V> s;
   size_t off = 0;
   auto take = [&](size_t bytes) {
@@ -377,7 +379,7 @@ template <typename V> __device__ Smem<V> carve(const Plan& P, const Bufs& B, uns
     s.tc = (double*)take(sizeof(double) * TT);
     s.te = (double*)take(sizeof(double) * TT);
   }
-  s.sct = (double2*)take(sizeof(double2) * (P.fixed64 ? 512 : 256));
+  s.sct = (double2*)take(sizeof(double2) * (F64 ? 512 : 256));
   s.red = (double*)take(sizeof(double) * THREADS * (3 * P.D + 5));
   s.fin = (double*)take(sizeof(double) * PSTRIDE);
   s.sc = (double*)take(sizeof(double) * SC_N);

@@ -54,7 +54,7 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
   using V = typename VT<T>::v;
   extern __shared__ __align__(16) unsigned char smem_raw[];
   __shared__ int sflag;
-  const Smem<V> S = carve<V>(P, B, smem_raw);
+  const Smem<V> S = carve<V, F64>(P, B, smem_raw);
   const int D = P.D;
   // an unreported error from an earlier launch makes every later launch a no-op
   if (__ldcg(B.status) != ST_OK) return;
@@ -66,8 +66,15 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
     sc[SC_P + threadIdx.x] = __ldcg(B.ctrl + 8 + threadIdx.x);
   }
   // passes on the integer units: tables in multiplier form, phases in turns
-  Smem<V> SB = S;  // for the table builds, which use the FP64 sincos table
-  if (F64) SB.sct = (double2*)B.sct;
+  auto build = [&](int what) {
+    if constexpr (F64) {
+      Smem<V> SB = S;  // the builds use the FP64 sincos table
+      SB.sct = (double2*)B.sct;
+      build_tables(P, B, SB, what);
+    } else {
+      build_tables(P, B, S, what);
+    }
+  };
   auto load = [&](int what) {
     if constexpr (F64) load_mult_tables(P, B, S, what);
     else load_tables(P, B, S, what);
@@ -95,7 +102,7 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
     }
     if (threadIdx.x < D) sc[SC_QN + threadIdx.x] = sc[SC_Q + threadIdx.x];
     __syncthreads();
-    build_tables(P, B, SB, TB_V);
+    build(TB_V);
     if (!grid_sync(B, &sflag)) return;
     load(LT_V);
     __syncthreads();
@@ -108,7 +115,7 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
     finish(B, S, 1, D + 1);
     centre_after_potential(P, S, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
-    build_tables(P, B, SB, TB_A);
+    build(TB_A);
     if (!grid_sync(B, &sflag)) return;
     load(LT_A);
     __syncthreads();
@@ -143,7 +150,7 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
     finish(B, S, 0, D + 1);
     centre_after_kinetic(P, S, RN.motion);
     if (sc[SC_ERR] != 0.0) goto done;
-    build_tables(P, B, SB, TB_K | (hasv ? TB_V : 0));
+    build(TB_K | (hasv ? TB_V : 0));
     if (!grid_sync(B, &sflag)) return;
     load(LT_K | (hasv ? LT_V : 0));
     if (threadIdx.x < D) sc[SC_Q + threadIdx.x] = sc[SC_QN + threadIdx.x];
@@ -166,7 +173,7 @@ __device__ __forceinline__ void propagate_body(const Plan& P, const Bufs& B, con
       finish(B, S, 1, D + 1);
       centre_after_potential(P, S, RN.motion);
       if (sc[SC_ERR] != 0.0) goto done;
-      build_tables(P, B, SB, TB_A);
+      build(TB_A);
       if (!grid_sync(B, &sflag)) return;
       load(LT_A);
       __syncthreads();

@@ -285,7 +285,7 @@ __device__ __forceinline__ BlockScale chunk_scale(ScanRec s, int* rec) {
 template <bool INV, int KIND, int DM = MAXD>
 __device__ __noinline__ int axis_pass64(const Plan& P, const Bufs& B, const PassArgs& A, int res_in) {
   using V = double2;
-  const Smem<V> S = carve<V>(P, B, smem_raw64);
+  const Smem<V> S = carve<V, true>(P, B, smem_raw64);
   const AxisPlan& ax = P.ax[A.l];
   const int n = ax.n, W = ax.W, D = P.D;
   const bool contig = (A.l == D - 1);
