@@ -9,11 +9,12 @@ is needed between iterations.  The roofline is stated against the FP64 FMA
 rate measured in the same run; the transforms run on the integer units as
 64-bit fixed point, so the fraction may exceed 1.
 
-Secondary lines (other keys of the same JSON line): the 256 x 256 atom-diatom
-workload, 3D harmonic 32^3, 16^8 FP32, mixed precision, batch, adjoint,
-convergence orders, an ensemble.
+One short JSON line is printed.  With --details PATH the secondary workloads
+run too (the 256 x 256 atom-diatom workload, 3D harmonic 32^3, 16^8 FP32, mixed
+precision, batch, adjoint, convergence orders, an ensemble), and the line's
+record, with its notes, and theirs are written to PATH.
 
-python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference]
+python bench.py [--gpus N] [--steps K] [--warmup W] [--impl ours|reference] [--details PATH]
 
 With N > 1 (torchrun) every rank runs an independent replica on its own GPU
 (the single-grid path has no data to exchange); value is the sum over ranks
@@ -1111,6 +1112,19 @@ def atom_diatom_leg(mg, torch, dev, args, flush):
             "error_vs_oracle": err, "cpu_baseline": cpu}
 
 
+LINE_LIMIT = 2800  # characters: readers of the output keep no more than its end
+
+
+def contract_line(record):
+    """The printed line: the record without the keys that explain the numbers,
+    which stay in the details."""
+    line = dict(record)
+    line["roofline"] = {k: record["roofline"][k] for k in ("bound", "achieved", "peak", "unit", "frac", "traffic", "kernel")}
+    line["roofline"]["hbm"] = {k: record["roofline"]["hbm"][k] for k in ("achieved", "peak", "unit", "frac")}
+    line["e2e"] = {k: v for k, v in record["e2e"].items() if k != "note"}
+    return json.dumps(line)
+
+
 def main():
     ap = argparse.ArgumentParser()
     ap.add_argument("--gpus", type=int, default=1)
@@ -1121,7 +1135,8 @@ def main():
                     help="only the warm-up and timed propagate calls, as in the timed region (for ncu captures)")
     ap.add_argument("--profile-case", default="hh8_fp64",
                     choices=["hh8_fp64", "atom_diatom", "hh7_fp32", "hh7_fp64", "tc_dft16"])
-    ap.add_argument("--headline-only", action="store_true", help="skip the secondary legs")
+    ap.add_argument("--details", metavar="PATH", help="run the secondary legs too and write the full record to PATH")
+    ap.add_argument("--headline-only", action="store_true", help="with --details: skip the secondary legs")
     args = ap.parse_args()
     if args.impl == "reference":
         return run_reference(args)
@@ -1232,7 +1247,7 @@ def main():
                                    f"(slowest {all_slowest:.1f} s)"}}
 
     secondary = {}
-    if not args.headline_only:
+    if args.details and not args.headline_only:
         flush = torch.empty(FLUSH_BYTES, dtype=torch.uint8, device=dev)
         secondary["atom_diatom_256"] = atom_diatom_leg(mg, torch, dev, args, flush)
         secondary["mixed_precision"] = mixed_precision_leg(mg, torch, dev, args, flush)
@@ -1277,8 +1292,10 @@ def main():
         "clocks": clk.summary(),
         "wall_s": wall,
     }
-    line.update(secondary)
-    print(json.dumps(line))
+    if args.details:
+        with open(args.details, "w") as f:
+            json.dump(dict(line, **secondary), f)
+    print(contract_line(line))
     if dist is not None:
         dist.destroy_process_group()
 
