@@ -6,8 +6,9 @@ the grid's shape, u = psi sqrt(prod dq)) from the grid centre (q0, p0), and
 returns (uT, qT, pT).  For the atom-diatom potential, theta = (Dm, a, beta, A)
 (float64 tensor) replaces those four parameters of the potential; other
 potentials take an empty theta.  The backward pass calls the reversible
-adjoint kernel: it regenerates the trajectory backwards instead of storing it,
-and leaves `prop` at the initial state.  Gradients follow PyTorch's complex
+adjoint kernel: it regenerates the trajectory backwards instead of storing it
+(to rounding: large grids propagate with other arithmetic units than the
+adjoint), and leaves `prop` at the initial state.  Gradients follow PyTorch's complex
 convention, dL/dRe u + i dL/dIm u, which is the cotangent mg_adjoint takes.
 
 The forward pass keeps its final state (uT, qT, pT) and the potential it ran

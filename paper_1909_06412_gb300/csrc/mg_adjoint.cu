@@ -7,7 +7,10 @@
 // dJ = Re sum conj(ubar) du + qbar.dq + pbar.dp.  There is no tape: each
 // substep is undone with the same substep at the negated time, which is exact
 // because the integrator is time-reversible (Sec. II.G).  The same passes
-// apply the substep's vector-Jacobian product.
+// apply the substep's vector-Jacobian product.  They run on the FP64 units;
+// where mg_propagate used the integer units (FP64 grids with many points per SM,
+// mg_rules.h), the trajectory regenerated here agrees with the forward one to
+// rounding.
 //
 // Potential substep u' = e^{-i s V/hbar} u, p' = p - s g
 // (eq:eom_pt_solution_case_III_V), with gbar = -s pbar':

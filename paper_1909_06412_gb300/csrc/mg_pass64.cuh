@@ -11,7 +11,7 @@
 // cycles of integer work and a butterfly's additions a few each.  What bounds
 // this pass is latency: long dependent chains at 8 warps an SM (a thread needs
 // up to 255 registers).  Measured per call, before -> after: 128^3 Duschinsky
-// 9.32 -> 6.72 ms, 128 x 2048 Secrest-Johnson 1.96 -> 1.68 ms.  512 threads
+// 9.32 -> 6.73 ms, 128 x 2048 Secrest-Johnson 1.96 -> 1.69 ms.  512 threads
 // (8.2, 1.81 ms) and two CTAs an SM (10.4 ms on 128^3) spill and lose.
 #pragma once
 #include <cuda_runtime.h>
@@ -259,7 +259,7 @@ struct ScanRec {
     q += fx_square(m, e);
   }
 };
-// The chunk's scale from every thread's record (all threads; two barriers).
+// The chunk's scale from every thread's record (all threads; one barrier).
 __device__ __forceinline__ BlockScale chunk_scale(ScanRec s, int* rec) {
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
   const int E = __reduce_max_sync(0xffffffffu, s.e);

@@ -28,8 +28,8 @@
 // line's coordinate from running sums of those), and one FP64 value per line
 // and moment is formed at the end of the line.
 //
-// Measured: a 12^8 yoshida4 step 785 -> 275 ms, a 12^4 suzuki4 call 3.96 ->
-// 2.01 ms against the same plan on the FP64 units.  What bounds it now is
+// Measured: a 12^8 yoshida4 step 785 -> 276 ms, a 12^4 suzuki4 call 3.96 ->
+// 2.06 ms against the same plan on the FP64 units.  What bounds it now is
 // latency: 12 (8) warps an SM at up to 168 (255) registers a thread issue 0.30
 // instructions a cycle and scheduler; the stalls are the teams' barriers
 // (24%), fixed-latency dependences (21%) and shared and global loads (18%).  18
